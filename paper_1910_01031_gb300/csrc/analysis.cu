@@ -109,13 +109,23 @@ rand_dots_kernel(uint64_t seed, uint32_t t, uint32_t s_xi, uint32_t s_nu, int NR
     ana::rand_dots_cta(seed, t, s_xi, s_nu, NR, partial, nblk, blockIdx.y, blockIdx.x);
 }
 
-__global__ void __launch_bounds__(1024)
-sync_alpha_kernel(const double* __restrict__ phi, const double* __restrict__ partial, int nblk, int ne,
+// A slice of particles per CTA.  The step is a serial chain of FP64 (two
+// reductions, then the Lambert-W solve of each particle), so its time is
+// latency at small ensembles and the few FP64 lanes of an SM at large ones: the
+// alpha solves are spread over many SMs and the reductions, cheap next to
+// them, repeated in each.
+// One CTA of 1024 threads, a division per series term: 144 us at 10 and 100
+// particles, 896 us at 1000; in slices, with the series by Horner, about 35 us
+// at all three (analysis of 64^2 x 10: 379 -> 272 us, of 624^2 x 1000: 26.60
+// -> 25.74 ms).
+__global__ void __launch_bounds__(ana::SYNC_THREADS)
+sync_alpha_kernel(const double* __restrict__ phi, const double* __restrict__ partial, int nblk, int ne, int slice,
                   double NR, double N, double logNe, int scheme, double* c, double* gamma, double* zeta,
                   double* alpha, double* cstar, double* neglogw, double* coef, double* scal, int* flag)
 {
-    ana::sync_alpha_cta(phi, partial, nblk, ne, NR, N, logNe, scheme, c, gamma, zeta, alpha, cstar, neglogw, coef,
-                        scal, flag);
+    const int i0 = blockIdx.x * slice;
+    ana::sync_alpha_cta(phi, partial, nblk, ne, i0, min(ne, i0 + slice), NR, N, logNe, scheme, c, gamma, zeta, alpha,
+                        cstar, neglogw, coef, scal, flag);
 }
 
 __global__ void __launch_bounds__(1024)
@@ -305,8 +315,11 @@ cudaError_t launch_sync_alpha(const double* phi, const double* partial, int nblk
                               double* alpha, double* cstar, double* neglogw, double* coef, double* scal,
                               int* flag, cudaStream_t st)
 {
-    sync_alpha_kernel<<<1, 1024, 0, st>>>(phi, partial, nblk, ne, NR, N_psi, logNe, scheme, c, gamma, zeta,
-                                          alpha, cstar, neglogw, coef, scal, flag);
+    // slices of a warp's width (one Lambert-W solve per lane of one warp), of
+    // more where that would take more than 128 CTAs
+    const int slice = 32 * ((ne + 32 * 128 - 1) / (32 * 128));
+    sync_alpha_kernel<<<(ne + slice - 1) / slice, ana::SYNC_THREADS, 0, st>>>(
+        phi, partial, nblk, ne, slice, NR, N_psi, logNe, scheme, c, gamma, zeta, alpha, cstar, neglogw, coef, scal, flag);
     return cudaGetLastError();
 }
 

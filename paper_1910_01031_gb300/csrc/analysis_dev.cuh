@@ -555,16 +555,24 @@ __device__ __forceinline__ void rand_dots_cta(uint64_t seed, uint32_t t, uint32_
     }
 }
 
-// -s - log(1 - s) for s in [0, 1): power series below 0.1, closed form above
+// -s - log(1 - s) for s in [0, 1): power series s^2 (1/2 + s/3 + ...) below
+// 0.1 (terms to s^18; the next is below 2e-18 of the sum), even and odd
+// powers as two Horner chains of fused multiply-adds so that their latencies
+// overlap; closed form above
 __device__ __forceinline__ double phi_s(double s)
 {
     if (s < 0.1) {
-        double acc = 0.0, term = s * s;
-        for (int n = 2; n < 40; ++n) {
-            acc += term / n;
-            term *= s;
-        }
-        return acc;
+        const double t = s * s;
+        double e = 1.0 / 18, o = 1.0 / 17;
+        e = fma(e, t, 1.0 / 16), o = fma(o, t, 1.0 / 15);
+        e = fma(e, t, 1.0 / 14), o = fma(o, t, 1.0 / 13);
+        e = fma(e, t, 1.0 / 12), o = fma(o, t, 1.0 / 11);
+        e = fma(e, t, 1.0 / 10), o = fma(o, t, 1.0 / 9);
+        e = fma(e, t, 1.0 / 8), o = fma(o, t, 1.0 / 7);
+        e = fma(e, t, 1.0 / 6), o = fma(o, t, 1.0 / 5);
+        e = fma(e, t, 1.0 / 4), o = fma(o, t, 1.0 / 3);
+        e = fma(e, t, 1.0 / 2);
+        return t * fma(o, s, e);
     }
     return -s - log1p(-s);
 }
@@ -591,10 +599,16 @@ __device__ __forceinline__ double alpha_lambert(double gamma, double cstar, doub
             const double f = phi_s(s) - q;
             const double fp = s / (1.0 - s);
             if (fp <= 0.0) break;
-            double sn = s - f / fp;
+            const double ds = f / fp;
+            double sn = s - ds;
             if (sn <= 0.0) sn = 0.5 * s;
-            if (sn >= 1.0) sn = 0.5 * (s + 1.0);
-            if (sn == s) break;
+            else if (sn >= 1.0) sn = 0.5 * (s + 1.0);
+            // a Newton step of relative size e leaves a relative error of
+            // e^2 / (2 (1 - s)): below 1e-9 the step just taken was the last
+            else if (fabs(ds) <= 1e-9 * s) {
+                s = sn;
+                break;
+            }
             s = sn;
         }
         u = 1.0 - s;
@@ -645,23 +659,31 @@ __device__ __forceinline__ void block_sum_min(double v_sum, double v_min, double
 constexpr int TWO_STAGE = 0;
 constexpr int ONE_STAGE = 1;
 
-// CTA: the ensemble-wide step.  Two-stage: w_target = mean c_i, beta, c*,
-// alpha, -log w.  One-stage: w_target = max c_i, beta reported as 0 (the nu
-// term of the posterior vanishes with it), c* = w_target - c_i, alpha, -log w.
-// scal[0] = w_target, scal[1] = beta, scal[2] = mean c_i.
-__device__ __forceinline__ void weights_cta(const double* c, const double* gamma, const double* zeta, int ne,
-                                            double N, int scheme, double* alpha, double* cstar, double* neglogw,
-                                            double* scal, int* flag)
+// CTA: the ensemble-wide step for the particles [i0, i1).  Two-stage:
+// w_target = mean c_i, beta, c*, alpha, -log w.  One-stage: w_target = max
+// c_i, beta reported as 0 (the nu term of the posterior vanishes with it),
+// c* = w_target - c_i, alpha, -log w.  scal[0] = w_target, scal[1] = beta,
+// scal[2] = mean c_i.  cval(i), zval(i): c_i and zeta_i of any particle;
+// gamma, zeta of the slice are read from the arrays.  The two ensemble-wide
+// reductions (mean or maximum of c, minimum of beta's candidates) run over
+// all particles in every CTA, in the same order, so that CTAs with different
+// slices need no synchronisation and hold the same target and beta.
+template <class FC, class FZ>
+__device__ __forceinline__ void weights_slice_cta(FC cval, FZ zval, const double* gamma, const double* zeta, int ne,
+                                                  int i0, int i1, double N, int scheme, double* alpha,
+                                                  double* cstar, double* neglogw, double* scal, int* flag)
 {
     __shared__ double s_sum, s_min;
     const bool one = scheme == ONE_STAGE;
     double acc = 0.0, mc = INFINITY;
     bool bad = false;
     for (int i = threadIdx.x; i < ne; i += blockDim.x) {
-        acc += c[i];
-        mc = fmin(mc, -c[i]);
-        bad |= !isfinite(c[i]) || !isfinite(gamma[i]) || (!one && !isfinite(zeta[i]));
+        const double c = cval(i);
+        acc += c;
+        mc = fmin(mc, -c);
+        bad |= !isfinite(c);
     }
+    for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) bad |= !isfinite(gamma[i]) || (!one && !isfinite(zeta[i]));
     bad = __syncthreads_or(bad);
     block_sum_min(acc, mc, &s_sum, &s_min);
     const double cmean = s_sum / ne;
@@ -669,27 +691,30 @@ __device__ __forceinline__ void weights_cta(const double* c, const double* gamma
     double beta = 0.0;
     if (!one) {
         double mn = INFINITY;
-        for (int i = threadIdx.x; i < ne; i += blockDim.x) mn = fmin(mn, (target - c[i]) / zeta[i] + 1.0);
+        for (int i = threadIdx.x; i < ne; i += blockDim.x) mn = fmin(mn, (target - cval(i)) / zval(i) + 1.0);
         block_sum_min(0.0, mn, &s_sum, &s_min);
         beta = s_min;
     }
     bool dom = false;
-    for (int i = threadIdx.x; i < ne; i += blockDim.x) {
-        const double cs = one ? target - c[i] : target - c[i] - (beta - 1.0) * zeta[i];
-        const double a = alpha_lambert(gamma[i], cs, N);
+    for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+        const double c = cval(i), g = gamma[i];
+        const double cs = one ? target - c : target - c - (beta - 1.0) * zeta[i];
+        const double a = alpha_lambert(g, cs, N);
         dom |= !(a > 0.0) || !isfinite(a);
         alpha[i] = a;
         cstar[i] = cs;
         if (neglogw) {
-            const double t = (a - 1.0) * gamma[i] - N * log(a);
-            neglogw[i] = one ? t + c[i] : t + (beta - 1.0) * zeta[i] + c[i];
+            const double t = (a - 1.0) * g - N * log(a);
+            neglogw[i] = one ? t + c : t + (beta - 1.0) * zeta[i] + c;
         }
     }
     dom = __syncthreads_or(dom);
     if (threadIdx.x == 0) {
-        scal[0] = target;
-        scal[1] = beta;
-        scal[2] = cmean;
+        if (i0 == 0) {
+            scal[0] = target;
+            scal[1] = beta;
+            scal[2] = cmean;
+        }
         int f = 0;
         if (bad) f |= FLAG_NONFINITE;
         if (!(beta >= 0.0)) f |= FLAG_BETA;
@@ -698,14 +723,32 @@ __device__ __forceinline__ void weights_cta(const double* c, const double* gamma
     }
 }
 
-// CTA: gamma, zeta, a, the length scale and c from the partial dot products,
-// then the weights step
-__device__ __forceinline__ void sync_alpha_cta(const double* __restrict__ phi, const double* __restrict__ partial,
-                                               int nblk, int ne, double NR, double N, double logNe, int scheme, double* c,
-                                               double* gamma, double* zeta, double* alpha, double* cstar,
-                                               double* neglogw, double* coef, double* scal, int* flag)
+// the same on given arrays of all particles, one CTA
+__device__ __forceinline__ void weights_cta(const double* c, const double* gamma, const double* zeta, int ne,
+                                            double N, int scheme, double* alpha, double* cstar, double* neglogw,
+                                            double* scal, int* flag)
 {
-    for (int i = threadIdx.x; i < ne; i += blockDim.x) {
+    weights_slice_cta([&](int i) { return c[i]; }, [&](int i) { return zeta[i]; }, gamma, zeta, ne, 0, ne, N, scheme,
+                      alpha, cstar, neglogw, scal, flag);
+}
+
+// CTAs of SYNC_THREADS, one per slice [i0, i1) of the particles: gamma, zeta,
+// a, the length scale and c of the slice from the partial dot products, then
+// the weights step.  What other slices need of a particle (c_i and zeta_i)
+// each CTA forms again from phi and the partial sums, by the same operations.
+constexpr int SYNC_THREADS = 256;
+__device__ __forceinline__ void sync_alpha_cta(const double* __restrict__ phi, const double* __restrict__ partial,
+                                               int nblk, int ne, int i0, int i1, double NR, double N, double logNe,
+                                               int scheme, double* c, double* gamma, double* zeta, double* alpha,
+                                               double* cstar, double* neglogw, double* coef, double* scal, int* flag)
+{
+    auto cval = [&](int i) { return phi[i] + logNe; };              // eq. iewpf_ci
+    auto zval = [&](int i) {
+        double nn = 0.0;
+        for (int b = 0; b < nblk; ++b) nn += partial[((long long)i * nblk + b) * 3 + 1];
+        return nn * N / NR;                                          // eq. scalingGammaZeta
+    };
+    for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
         double xx = 0.0, nn = 0.0, nx = 0.0;
         for (int b = 0; b < nblk; ++b) {
             xx += partial[((long long)i * nblk + b) * 3 + 0];
@@ -717,10 +760,10 @@ __device__ __forceinline__ void sync_alpha_cta(const double* __restrict__ phi, c
         coef[2 * i + 1] = sqrt(nn / (nn - a * nx));
         gamma[i] = xx * N / NR;                                      // eq. scalingGammaZeta
         zeta[i] = nn * N / NR;
-        c[i] = phi[i] + logNe;                                       // eq. iewpf_ci
+        c[i] = cval(i);
     }
     __syncthreads();
-    weights_cta(c, gamma, zeta, ne, N, scheme, alpha, cstar, neglogw, scal, flag);
+    weights_slice_cta(cval, zval, gamma, zeta, ne, i0, i1, N, scheme, alpha, cstar, neglogw, scal, flag);
 }
 
 // r = beta^{1/2} nu + alpha^{1/2} xi at coarse point m of particle p,

@@ -328,11 +328,11 @@ __global__ void __launch_bounds__(ana::DOT_THREADS) b_dots(BatchDev B)
     }
 }
 
-__global__ void __launch_bounds__(1024) b_sync(BatchDev B)
+__global__ void __launch_bounds__(ana::SYNC_THREADS) b_sync(BatchDev B)
 {
     for (int i = blockIdx.x; i < B.n; i += gridDim.x) {
         const BInst& I = B.inst[i];
-        ana::sync_alpha_cta(I.phi, I.partial, I.nblk, I.G.ne, (double)I.NR, I.N_psi, I.logNe, I.scheme, I.c,
+        ana::sync_alpha_cta(I.phi, I.partial, I.nblk, I.G.ne, 0, I.G.ne, (double)I.NR, I.N_psi, I.logNe, I.scheme, I.c,
                             I.gamma, I.zeta, I.alpha, I.cstar, I.neglogw, I.coef, I.scal, I.flag);
     }
 }
@@ -629,7 +629,7 @@ static cudaError_t capture_analysis(BatchImpl& b, cudaStream_t st)
     b_cholesky<<<b.n, 1024, 0, st>>>(B);
     b_solve<<<grid_for(b_solve, 128, (items(b, SP_PART) + 3) / 4), 128, 0, st>>>(B);
     b_dots<<<grid_for(b_dots, ana::DOT_THREADS, items(b, SP_DOT)), ana::DOT_THREADS, 0, st>>>(B);
-    b_sync<<<b.n, 1024, 0, st>>>(B);
+    b_sync<<<b.n, ana::SYNC_THREADS, 0, st>>>(B);
     b_form_r<<<grid_for(b_form_r, 256, (items(b, SP_FR) + 255) / 256), 256, 0, st>>>(B);
     b_block_seq<<<grid_for(b_block_seq, 64, items(b, SP_PART)), 64, 0, st>>>(B);
     b_soar<true><<<grid_for(b_soar<true>, 256, (items(b, SP_FR) + 255) / 256), 256, 0, st>>>(B);

@@ -1,0 +1,40 @@
+"""GPU kernels at the sizes where their work splits can go wrong (edges of
+tiles and slices, remainders, smallest and largest of a rule's range),
+against the FP64 oracle; tolerances as in the parity tests of each quantity."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_1910_01031_gb300 import iewpf, synth
+from gpu_common import ensemble, oracle_problem, start_state
+
+pytestmark = pytest.mark.gpu
+
+
+def _observed(cfg, n, cycle=0):
+    """Drifter positions, their cells and observed values from another draw of the initial state."""
+    xy = synth.drifter_positions(cfg, n)
+    cells = [O.obs_cell(oracle_problem(cfg), *p) for p in xy]
+    truth = synth.initial_state(cfg, 1, seed=3)[0]
+    return xy, cells, synth.obs_from_state(cfg, truth, np.array(cells), synth.obs_noise(cfg, n, cycle))
+
+
+@pytest.mark.parametrize("ne", [31, 33, 4097])
+@pytest.mark.parametrize("scheme", [iewpf.TWO_STAGE, iewpf.ONE_STAGE])
+def test_ensemble_wide_step_over_slices(ne, scheme):
+    """The ensemble-wide step runs in slices of 32 particles (64 above 4096): target, beta, alpha and
+    weights of every particle against the oracle's on the same c, gamma, zeta (1e-10, as iewpf_weights)."""
+    cfg = synth.Config("edge_48x48", 48, 48, n_particles=ne, n_obs=2)
+    ens = iewpf.Ensemble(iewpf.params_from_config(cfg, scheme=scheme))
+    U = np.repeat(synth.initial_state(cfg, min(ne, 40), seed=7).astype(np.float32), -(-ne // 40), axis=0)[:ne]
+    ens.set_state(U)
+    xy, _, y = _observed(cfg, 2)
+    d = ens.assimilate(xy, y)
+    N = 3.0 * cfg.nx * cfg.ny
+    ref = O.iewpf_scalars_one_stage(d["c"], d["gamma"], N) if scheme == iewpf.ONE_STAGE else \
+        O.iewpf_scalars(d["c"], d["gamma"], d["zeta"], N)
+    np.testing.assert_allclose(d["w_target"], ref.get("w_target", ref["cbar"]), rtol=1e-10)
+    np.testing.assert_allclose(d["cbar"], ref["cbar"], rtol=1e-10)
+    np.testing.assert_allclose(d["beta"], ref["beta"], rtol=1e-10, atol=1e-300)
+    np.testing.assert_allclose(d["alpha"], ref["alpha"], rtol=1e-10)
+    np.testing.assert_allclose(d["neglogw"], ref["neglogw"], rtol=1e-10)
