@@ -139,8 +139,8 @@ __global__ void form_r_kernel(uint64_t seed, uint32_t t, uint32_t s_xi, uint32_t
                               const double* __restrict__ coef, const double* __restrict__ scal,
                               const double* __restrict__ alpha, float* __restrict__ r)
 {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m < NR) ana::form_r_one(seed, t, s_xi, s_nu, NR, coef, scal, alpha, r, blockIdx.y, m);
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (4 * q < NR) ana::form_r_block(seed, t, s_xi, s_nu, NR, coef, scal, alpha, r, blockIdx.y, q);
 }
 
 __global__ void block_seq_kernel(float* __restrict__ r, int NR, const float* __restrict__ M49,
@@ -335,7 +335,7 @@ cudaError_t launch_form_r(uint64_t seed, uint32_t t, uint32_t s_xi, uint32_t s_n
                           const double* coef, const double* scal, const double* alpha, float* r,
                           cudaStream_t st)
 {
-    dim3 grid((NR + 255) / 256, ne);
+    dim3 grid(((NR + 3) / 4 + 255) / 256, ne);
     form_r_kernel<<<grid, 256, 0, st>>>(seed, t, s_xi, s_nu, NR, coef, scal, alpha, r);
     return cudaGetLastError();
 }

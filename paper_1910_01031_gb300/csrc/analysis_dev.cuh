@@ -492,34 +492,60 @@ __device__ __forceinline__ void solve_levels_warp(const double* __restrict__ L, 
 constexpr int DOT_THREADS = 256;
 constexpr int DOT_BLOCKS_PER_CTA = 8;
 
-// CTA of DOT_THREADS: partial sums of xi^T xi, nu~^T nu~, nu~^T xi (FP64
-// normals) of particle p over the Philox blocks of slice bx
+// u = (a + 1/2) 2^-32 in one FP64 operation: the bits of 2^20 + a 2^-32 are a
+// under a fixed upper word, and the difference is exact
+__device__ __forceinline__ double uniform64(uint32_t a)
+{
+    return __hiloint2double(0x41300000, (int)a) - (0x1p20 - 0x1p-33);
+}
+
+// log u in FP32 to float precision over all of (0, 1), next to 1 as well (see box_muller32)
+__device__ __forceinline__ float log_uniform32(uint32_t a)
+{
+    return a < 0x80000000u ? logf(((float)a + 0.5f) * 0x1p-32f) : log1pf(-(((float)(~a) + 0.5f) * 0x1p-32f));
+}
+
+// CTA of DOT_THREADS: partial sums of xi^T xi, nu~^T nu~, nu~^T xi of particle
+// p over the Philox blocks of slice bx, from the Box-Muller identities: with
+// z = r (cos, sin)(pi 2u_b), r^2 = -2 log u_a, a pair adds -2 log u_a to the
+// squared norm and, with the pair of the other vector, r_nu r_xi cos(pi
+// (2u_b,nu - 2u_b,xi)) to the cross product.
+//  * Squared norms in FP64: sum log u = log prod u, a product of the thread's
+//    uniforms (at most 16, each at least 2^-33, so far from underflow) and
+//    one logarithm for all of them: two FP64 operations per pair instead of a
+//    logarithm each, on the few FP64 lanes that bound this kernel.
+//  * The cross product sets only the projection coefficient a of eq.
+//    nuPerpendicular, not gamma or zeta: its terms are formed in FP32, the
+//    angle's difference in 32-bit integers, where its period is exact, and
+//    summed with their rounding errors (two-sum) until the thread's FP64 total.
+//    A term's rms error against 64 bits is 0.84e-7, 1.10e-7 when the difference
+//    was rounded to FP32 unreduced and the logarithms taken in FP64.
+// With form_r_block 4.05 ms per 1000 x 208^2 coarse points with an FP64
+// logarithm per pair and a generator per normal, 0.57 ms so.
 __device__ __forceinline__ void rand_dots_cta(uint64_t seed, uint32_t t, uint32_t s_xi, uint32_t s_nu, int NR,
                                               double* __restrict__ partial, int nblk, int p, int bx)
 {
     const uint2 key = seed_key(seed);
     const int nq = (NR + 3) / 4;
-    double xx = 0.0, nn = 0.0, nx = 0.0;
+    double px = 1.0, pn = 1.0;                       // products of the u_a of xi and of nu~
+    double tx = 0.0, tn = 0.0, tc = 0.0;             // terms of the last, partial block
+    float cs = 0.0f, ce = 0.0f;                      // cross product: sum and its rounding errors
+    static_assert(2 * DOT_BLOCKS_PER_CTA * 33 < 1000, "the products stay normal");
     for (int b = bx * DOT_THREADS + threadIdx.x; b < nq; b += nblk * DOT_THREADS) {
         const uint4 wx = philox4x32_10(make_uint4((uint32_t)b, (uint32_t)p, t, s_xi), key);
         const uint4 wn = philox4x32_10(make_uint4((uint32_t)b, (uint32_t)p, t, s_nu), key);
         if (4 * b + 3 < NR) {
-            // whole Box-Muller pairs: with z = r (cos, sin)(pi 2u_b) the pair
-            // contributes r^2 = -2 log u_a to the squared norm, and to the cross
-            // product r_nu r_xi cos(pi (2u_b,nu - 2u_b,xi)); one logarithm per
-            // pair, one square root and one cosine per pair of pairs
+            px *= uniform64(wx.x) * uniform64(wx.z);
+            pn *= uniform64(wn.x) * uniform64(wn.z);
             const uint32_t xa[2] = {wx.x, wx.z}, xb[2] = {wx.y, wx.w}, na[2] = {wn.x, wn.z}, nb[2] = {wn.y, wn.w};
 #pragma unroll
             for (int l = 0; l < 2; ++l) {
-                const double rx2 = -2.0 * log(((double)xa[l] + 0.5) * 0x1p-32);
-                const double rn2 = -2.0 * log(((double)na[l] + 0.5) * 0x1p-32);
-                const double d = ((double)nb[l] - (double)xb[l]) * 0x1p-31;   // 2u_b,nu - 2u_b,xi, exact
-                xx += rx2;
-                nn += rn2;
-                // nu~^T xi sets only the projection coefficient a of eq.
-                // nuPerpendicular, not gamma or zeta: its terms are formed in
-                // FP32 and summed in FP64
-                nx += (double)(sqrtf((float)(rx2 * rn2)) * cospif((float)d));
+                const float r = sqrtf(4.0f * log_uniform32(xa[l]) * log_uniform32(na[l]));
+                const float c = cospif((float)(int)(nb[l] - xb[l]) * 0x1p-31f);
+                const float v = r * c, ve = fmaf(r, c, -v);
+                const float s = cs + v, bb = s - cs;
+                ce += ((cs - (s - bb)) + (v - bb)) + ve;
+                cs = s;
             }
         } else {
             double x[4], v[4];
@@ -530,17 +556,17 @@ __device__ __forceinline__ void rand_dots_cta(uint64_t seed, uint32_t t, uint32_
 #pragma unroll
             for (int l = 0; l < 4; ++l) {
                 if (4 * b + l < NR) {
-                    xx = fma(x[l], x[l], xx);
-                    nn = fma(v[l], v[l], nn);
-                    nx = fma(v[l], x[l], nx);
+                    tx = fma(x[l], x[l], tx);
+                    tn = fma(v[l], v[l], tn);
+                    tc = fma(v[l], x[l], tc);
                 }
             }
         }
     }
     __shared__ double red[3][DOT_THREADS / 32];
-    xx = warp_sum(xx);
-    nn = warp_sum(nn);
-    nx = warp_sum(nx);
+    const double xx = warp_sum(fma(-2.0, log(px), tx));
+    const double nn = warp_sum(fma(-2.0, log(pn), tn));
+    const double nx = warp_sum(((double)cs + (double)ce) + tc);
     __syncthreads();
     if ((threadIdx.x & 31) == 0) {
         red[0][threadIdx.x >> 5] = xx;
@@ -766,20 +792,36 @@ __device__ __forceinline__ void sync_alpha_cta(const double* __restrict__ phi, c
     weights_slice_cta(cval, zval, gamma, zeta, ne, i0, i1, N, scheme, alpha, cstar, neglogw, scal, flag);
 }
 
-// r = beta^{1/2} nu + alpha^{1/2} xi at coarse point m of particle p,
-// nu = s (nu~ - a xi)
-__device__ __forceinline__ void form_r_one(uint64_t seed, uint32_t t, uint32_t s_xi, uint32_t s_nu, int NR,
-                                           const double* __restrict__ coef, const double* __restrict__ scal,
-                                           const double* __restrict__ alpha, float* __restrict__ r, int p, int m)
+// r = beta^{1/2} nu + alpha^{1/2} xi at the four coarse points of Philox block
+// q of particle p, nu = s (nu~ - a xi).  One thread per block: a block holds
+// four normals (the numbers normal32 returns one by one), so a thread per
+// point would run every generator four times.
+__device__ __forceinline__ void form_r_block(uint64_t seed, uint32_t t, uint32_t s_xi, uint32_t s_nu, int NR,
+                                             const double* __restrict__ coef, const double* __restrict__ scal,
+                                             const double* __restrict__ alpha, float* __restrict__ r, int p, int q)
 {
     const uint2 key = seed_key(seed);
-    const float xi = normal32(key, (uint32_t)p, t, s_xi, (uint32_t)m);
-    const float nut = normal32(key, (uint32_t)p, t, s_nu, (uint32_t)m);
+    const uint4 wx = philox4x32_10(make_uint4((uint32_t)q, (uint32_t)p, t, s_xi), key);
+    const uint4 wn = philox4x32_10(make_uint4((uint32_t)q, (uint32_t)p, t, s_nu), key);
+    float xi[4], nut[4], v[4];
+    box_muller32(wx.x, wx.y, xi[0], xi[1]);
+    box_muller32(wx.z, wx.w, xi[2], xi[3]);
+    box_muller32(wn.x, wn.y, nut[0], nut[1]);
+    box_muller32(wn.z, wn.w, nut[2], nut[3]);
     const float a = (float)coef[2 * p], sc = (float)coef[2 * p + 1];
     // square roots in FP32 (the factors enter an FP32 field; an FP64 square
-    // root per coarse point would cost more than the rest of the kernel)
+    // root per block would cost more than the rest of the kernel)
     const float sb = sqrtf((float)fmax(scal[1], 0.0)), sa = sqrtf((float)alpha[p]);
-    r[(long long)p * NR + m] = fmaf(sb, sc * fmaf(-a, xi, nut), sa * xi);
+#pragma unroll
+    for (int l = 0; l < 4; ++l) v[l] = fmaf(sb, sc * fmaf(-a, xi[l], nut[l]), sa * xi[l]);
+    float* __restrict__ o = r + (long long)p * NR + 4LL * q;
+    if ((NR & 3) == 0) {
+        *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+        for (int l = 0; l < 4; ++l)
+            if (4 * q + l < NR) o[l] = v[l];
+    }
 }
 
 // CTA of at least 64 threads: the 7x7 block roots of every observation of

@@ -37,7 +37,7 @@ enum Space : int {
     SP_HQ,         // entries of HQH^T
     SP_DOT,        // dot-product slices: particle x slice
     SP_FR,         // particle x coarse point
-    SP_NRM,        // particle x Philox block of the coarse normals
+    SP_NRM,        // particle x Philox block of the coarse normals and of the posterior field
     SP_FTILE,      // model-error fine tiles (FINE_TX x FINE_TY): particle x tile
     SP_COUNT
 };
@@ -339,13 +339,13 @@ __global__ void __launch_bounds__(ana::SYNC_THREADS) b_sync(BatchDev B)
 
 __global__ void b_form_r(BatchDev B)
 {
-    const long long* pre = space(B, SP_FR);
+    const long long* pre = space(B, SP_NRM);
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < pre[B.n]; q += (long long)gridDim.x * blockDim.x) {
         const int i = find_inst(pre, B.n, q);
         const BInst& I = B.inst[i];
-        const long long r = q - pre[i];
-        ana::form_r_one(I.seed, *I.cycle, I.stream_base + 1, I.stream_base + 2, (int)I.NR, I.coef, I.scal, I.alpha, I.r,
-                        (int)(r / I.NR), (int)(r % I.NR));
+        const long long nq = (I.NR + 3) / 4, r = q - pre[i];
+        ana::form_r_block(I.seed, *I.cycle, I.stream_base + 1, I.stream_base + 2, (int)I.NR, I.coef, I.scal, I.alpha,
+                          I.r, (int)(r / nq), (int)(r % nq));
     }
 }
 
@@ -630,7 +630,7 @@ static cudaError_t capture_analysis(BatchImpl& b, cudaStream_t st)
     b_solve<<<grid_for(b_solve, 128, (items(b, SP_PART) + 3) / 4), 128, 0, st>>>(B);
     b_dots<<<grid_for(b_dots, ana::DOT_THREADS, items(b, SP_DOT)), ana::DOT_THREADS, 0, st>>>(B);
     b_sync<<<b.n, ana::SYNC_THREADS, 0, st>>>(B);
-    b_form_r<<<grid_for(b_form_r, 256, (items(b, SP_FR) + 255) / 256), 256, 0, st>>>(B);
+    b_form_r<<<grid_for(b_form_r, 256, (items(b, SP_NRM) + 255) / 256), 256, 0, st>>>(B);
     b_block_seq<<<grid_for(b_block_seq, 64, items(b, SP_PART)), 64, 0, st>>>(B);
     b_soar<true><<<grid_for(b_soar<true>, 256, (items(b, SP_FR) + 255) / 256), 256, 0, st>>>(B);
     b_fine<true><<<grid_for(b_fine<true>, NTHREADS, items(b, SP_TILE)), NTHREADS, 0, st>>>(B);

@@ -6,7 +6,7 @@ import pytest
 
 from oracle import oracle as O
 from paper_1910_01031_gb300 import iewpf, synth
-from gpu_common import ensemble, oracle_problem, start_state
+from gpu_common import ensemble, oracle_problem, rel_l2, start_state
 
 pytestmark = pytest.mark.gpu
 
@@ -38,3 +38,20 @@ def test_ensemble_wide_step_over_slices(ne, scheme):
     np.testing.assert_allclose(d["beta"], ref["beta"], rtol=1e-10, atol=1e-300)
     np.testing.assert_allclose(d["alpha"], ref["alpha"], rtol=1e-10)
     np.testing.assert_allclose(d["neglogw"], ref["neglogw"], rtol=1e-10)
+
+
+@pytest.mark.parametrize("nx,ny", [(48, 48), (51, 48), (51, 51), (51, 57), (54, 57), (150, 141), (384, 375)])
+def test_random_vectors_over_philox_blocks(nx, ny):
+    """Coarse grids of every remainder modulo 4 (the last Philox block partly used) and of one and several
+    slices of the dot products: gamma and zeta at 1e-10, the state (which carries the projection of nu~
+    and the posterior field) at 1e-5."""
+    cfg = synth.Config("edge", nx, ny, n_particles=3, n_obs=1)
+    ens, P = ensemble(cfg), oracle_problem(cfg)
+    U32, U64 = start_state(cfg, 3)
+    ens.set_state(U32)
+    xy, cells, y = _observed(cfg, 1)
+    d = ens.assimilate(xy, y)
+    ref, dref = O.assimilate(P, U64, cells, y, t=0)
+    np.testing.assert_allclose(d["gamma"], dref["gamma"], rtol=1e-10)
+    np.testing.assert_allclose(d["zeta"], dref["zeta"], rtol=1e-10)
+    assert rel_l2(ens.get_state(), ref) <= 1e-5
