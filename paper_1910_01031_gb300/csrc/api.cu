@@ -396,15 +396,16 @@ cudaError_t launch_step(iewpf_ctx* ctx, int s)
     return launch_rk2_march(ctx->buf[0], ctx->buf[1], ctx->par, ctx->nsub, ctx->dtp, s, ctx->G, ctx->shape, ctx->st);
 }
 
-// Time every candidate shape of the marching kernel on the context's own
-// problem and keep the fastest.  A probe launch reads the current state and
-// writes the other buffer without flipping the parity, so the state is left
-// as it was; all shapes compute identical values.
+// Time candidate shapes of the marching kernel on the context's own problem
+// and keep the fastest: both kinds with 2 and 3 columns per lane (4 spill the
+// paired form and were never the fastest) over equal chunks of the rows (march_rows: the
+// last chunk as long as the others, down to a few rows for problems too small
+// to fill the GPU otherwise), then the warps per CTA of the best.  A probe
+// launch reads the current state and writes the other buffer without flipping
+// the parity, so the state is left as it was; all shapes compute identical
+// values.
 int tune_stepper(iewpf_ctx* ctx)
 {
-    static const int ncs[] = {2, 3, 4};
-    static const int ths[] = {16, 32, 64, 128, 256, 512};
-    static const int wps[] = {2, 4, 8};
     std::vector<int> ones(ctx->G.ne, 1);
     std::vector<float> dts(ctx->G.ne, (float)(ctx->P.dt_model / 16.0));
     CK(cudaMemcpyAsync(ctx->nsub, ones.data(), sizeof(int) * ones.size(), cudaMemcpyHostToDevice, ctx->st));
@@ -414,30 +415,33 @@ int tune_stepper(iewpf_ctx* ctx)
     CK(cudaEventCreate(&b));
     float best = 1e30f;
     MarchShape best_shape = ctx->shape;
-    for (int paired = 0; paired < 2; ++paired)
-    for (int nc : ncs)
-        for (int th : ths) {
-            if (th > 2 * ctx->G.ny || (paired && nc == 4)) continue;
-            for (int w : wps) {
-                MarchShape sh{nc, th, w, paired};
-                CK(launch_rk2_march(ctx->buf[0], ctx->buf[1], ctx->par, ctx->nsub, ctx->dtp, 0, ctx->G, sh, ctx->st));
-                CK(cudaEventRecord(a, ctx->st));
-                for (int r = 0; r < 3; ++r)
-                    CK(launch_rk2_march(ctx->buf[0], ctx->buf[1], ctx->par, ctx->nsub, ctx->dtp, 0, ctx->G, sh,
-                                        ctx->st));
-                CK(cudaEventRecord(b, ctx->st));
-                CK(cudaEventSynchronize(b));
-                float ms = 0.0f;
-                CK(cudaEventElapsedTime(&ms, a, b));
-                ctx->launches += 4;
-                if (ms < best) {
-                    best = ms;
-                    best_shape = sh;
-                }
-            }
+    auto probe = [&](const MarchShape& sh) -> int {
+        CK(launch_rk2_march(ctx->buf[0], ctx->buf[1], ctx->par, ctx->nsub, ctx->dtp, 0, ctx->G, sh, ctx->st));
+        CK(cudaEventRecord(a, ctx->st));
+        for (int r = 0; r < 3; ++r)
+            CK(launch_rk2_march(ctx->buf[0], ctx->buf[1], ctx->par, ctx->nsub, ctx->dtp, 0, ctx->G, sh, ctx->st));
+        CK(cudaEventRecord(b, ctx->st));
+        CK(cudaEventSynchronize(b));
+        float ms = 0.0f;
+        CK(cudaEventElapsedTime(&ms, a, b));
+        ctx->launches += 4;
+        if (ms < best) {
+            best = ms;
+            best_shape = sh;
         }
+        return IEWPF_OK;
+    };
+    int rc = IEWPF_OK;
+    for (int paired = 0; paired < 2 && !rc; ++paired)
+        for (int nc = 2; nc <= 3 && !rc; ++nc)
+            for (int th : march_rows(ctx->G.ny))
+                if ((rc = probe(MarchShape{nc, th, 4, paired}))) break;
+    const MarchShape at4 = best_shape;
+    for (int w : {2, 8})
+        if (!rc) rc = probe(MarchShape{at4.nc, at4.TH, w, at4.paired});
     cudaEventDestroy(a);
     cudaEventDestroy(b);
+    if (rc) return rc;
     ctx->shape = best_shape;
     ctx->stepper = 1 + best_shape.paired;
     ctx->tuned = true;
@@ -776,18 +780,15 @@ int iewpf_create(const iewpf_params_t* params, const double* mooring_xy, iewpf_c
     G.theta = (float)P.theta;
     G.inv_dx = (float)(1.0 / P.dx);
     G.inv_dy = (float)(1.0 / P.dy);
-    G.fdx = (float)(P.f * P.dx);
     G.fdy = (float)(P.f * P.dy);
-    G.fdx_half = (float)(0.5 * P.f * P.dx);
-    G.fdy_half = (float)(0.5 * P.f * P.dy);
-    G.inv_2g = (float)(0.5 / P.g);
     G.sgh = (float)(P.g * P.H_eq / P.f);
     G.inv_2dx = (float)(0.5 / P.dx);
     G.inv_2dy = (float)(0.5 / P.dy);
     G.theta2 = 2.0f * G.theta;
-    G.fdx2 = 2.0f * G.fdx;
-    G.fdy2 = 2.0f * G.fdy;
-    G.inv_4g = 0.5f * G.inv_2g;
+    G.fdx_2g = (float)(0.5 * P.f * P.dx / P.g);
+    G.fdy_2g = (float)(0.5 * P.f * P.dy / P.g);
+    G.dy_dx = (float)(P.dy / P.dx);
+    G.sqrt_g = (float)std::sqrt(P.g);
     G.g_half = 0.5f * G.g;
     G.gH = (float)(P.g * P.H_eq);
     G.ne = P.n_particles;

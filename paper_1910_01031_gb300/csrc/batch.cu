@@ -119,21 +119,23 @@ __global__ void b_nsub(BatchDev B)
     }
 }
 
-template <int NC, bool PAIRED>
-__global__ void __launch_bounds__(256) b_step(BatchDev B)
+template <int NC, bool RING, bool PAIRED>
+__global__ void __launch_bounds__(NC == 2 ? 384 : 256) b_step(BatchDev B)
 {
     const long long* pre = space(B, SP_STEP);
     const int s = *B.s;
-    const long long wpg = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < pre[B.n]; w += wpg) {
+    const long long wpg = (long long)gridDim.x * (blockDim.x >> 5);
+    // (the warp's index from lane 0: uniform, see rk2_march_kernel)
+    for (long long w = (long long)blockIdx.x * (blockDim.x >> 5) + __shfl_sync(march::FULL, (int)(threadIdx.x >> 5), 0);
+         w < pre[B.n]; w += wpg) {
         const int i = find_inst(pre, B.n, w);
         const march::StepArgs a = B.inst[i].step;     // by value: no reloads after the state stores
         const long long r = w - pre[i];
         const long long per_p = (long long)a.n_strips * a.n_chunks;
         const int p = (int)(r / per_p);
         const int rem = (int)(r % per_p);
-        if (PAIRED) march::march_warp_paired<NC>(a, p, rem / a.n_strips, rem % a.n_strips, s);
-        else march::march_warp<NC>(a, p, rem / a.n_strips, rem % a.n_strips, s);
+        if (PAIRED) march::march_warp_paired<NC, RING>(a, p, rem / a.n_strips, rem % a.n_strips, s);
+        else march::march_warp<NC, RING>(a, p, rem / a.n_strips, rem % a.n_strips, s);
     }
 }
 
@@ -412,6 +414,7 @@ struct BatchImpl {
     bool fgraph_err = false;
     int nc = 2;
     int warps = 4;
+    bool ring = false;  // every row held by one ring of lanes (march::ring)
     int paired = 0;     // scheme step with the two stages in f32x2 pairs (nc 2 or 3)
     int fixed = 0;
     bool tuned = false;
@@ -436,13 +439,12 @@ cudaError_t launch_step_nc(BatchImpl& b, cudaStream_t st)
         const int g = (int)std::min<long long>(need, resident_blocks((const void*)kern, thr));
         kern<<<g, thr, 0, st>>>(B);
     };
-    if (b.paired) {
-        if (b.nc == 2) run(b_step<2, true>);
-        else run(b_step<3, true>);
+    if (b.nc == 2) {
+        if (b.ring) b.paired ? run(b_step<2, true, true>) : run(b_step<2, true, false>);
+        else b.paired ? run(b_step<2, false, true>) : run(b_step<2, false, false>);
     } else {
-        if (b.nc == 2) run(b_step<2, false>);
-        else if (b.nc == 3) run(b_step<3, false>);
-        else run(b_step<4, false>);
+        if (b.ring) b.paired ? run(b_step<3, true, true>) : run(b_step<3, true, false>);
+        else b.paired ? run(b_step<3, false, true>) : run(b_step<3, false, false>);
     }
     return cudaGetLastError();
 }
@@ -458,16 +460,19 @@ int grid_for(K kern, int threads, long long work_items_per_block_units)
 
 cudaError_t batch_set_step_shape(BatchImpl& b, int nc, int th, int warps, int paired)
 {
-    if (paired && nc == 4) return cudaErrorInvalidValue;
+    if (nc != 2 && nc != 3) return cudaErrorInvalidValue;
     b.nc = nc;
     b.warps = warps;
     b.paired = paired;
+    // the ring form of the march when every problem's rows fit it (one kernel
+    // serves all problems)
+    b.ring = true;
+    for (int i = 0; i < b.n; ++i) b.ring = b.ring && march::ring(b.h_inst[i].G.nx, nc);
     long long acc = 0;
     for (int i = 0; i < b.n; ++i) {
         BInst& I = b.h_inst[i];
-        const int wuse = 32 * nc - 8;
         I.step.TH = th;
-        I.step.n_strips = (I.G.nx + wuse - 1) / wuse;
+        I.step.n_strips = b.ring ? 1 : (I.G.nx + 32 * nc - 9) / (32 * nc - 8);
         I.step.n_chunks = (I.G.ny + th - 1) / th;
         b.pre[(size_t)SP_STEP * (b.n + 1) + i] = acc;
         acc += (long long)I.step.n_strips * I.step.n_chunks * I.G.ne;
@@ -732,9 +737,10 @@ cudaError_t batch_forecast(BatchImpl& b, int n_steps, bool err, cudaStream_t st,
 // buffer without flipping the parity).
 cudaError_t batch_tune(BatchImpl& b, cudaStream_t st)
 {
-    static const int ncs[] = {2, 3, 4};
-    static const int ths[] = {32, 64, 128, 256, 512};
-    static const int wps[] = {2, 4, 8};
+    // chunk lengths: those of the tallest grid
+    int ny = 0;
+    for (const BInst& I : b.h_inst) ny = std::max(ny, I.G.ny);
+    const std::vector<int> ths = march_rows(ny);
     cudaError_t e;
     // every particle one probe step of dt_model / 16
     b.fixed = 16;
@@ -749,28 +755,36 @@ cudaError_t batch_tune(BatchImpl& b, cudaStream_t st)
     cudaEventCreate(&z);
     float best = 1e30f;
     int bnc = 2, bth = 64, bw = 4, bp = 0;
+    auto probe = [&](int nc, int th, int w, int paired) -> cudaError_t {
+        cudaError_t r;
+        if ((r = batch_set_step_shape(b, nc, th, w, paired)) != cudaSuccess) return r;
+        if ((r = launch_step_nc(b, st)) != cudaSuccess) return r;
+        cudaEventRecord(a, st);
+        if ((r = launch_step_nc(b, st)) != cudaSuccess) return r;
+        cudaEventRecord(z, st);
+        cudaEventSynchronize(z);
+        float ms = 0.0f;
+        cudaEventElapsedTime(&ms, a, z);
+        b.launches += 2;
+        if (ms < best) {
+            best = ms;
+            bnc = nc;
+            bth = th;
+            bw = w;
+            bp = paired;
+        }
+        return cudaSuccess;
+    };
+    // shapes as in the one-problem tuner: kinds, columns and chunks, then the warps of the best
     for (int paired = 0; paired < 2; ++paired)
-    for (int nc : ncs)
-        for (int th : ths)
-            for (int w : wps) {
-                if (paired && nc == 4) continue;
-                if ((e = batch_set_step_shape(b, nc, th, w, paired)) != cudaSuccess) return e;
-                if ((e = launch_step_nc(b, st)) != cudaSuccess) return e;
-                cudaEventRecord(a, st);
-                if ((e = launch_step_nc(b, st)) != cudaSuccess) return e;
-                cudaEventRecord(z, st);
-                cudaEventSynchronize(z);
-                float ms = 0.0f;
-                cudaEventElapsedTime(&ms, a, z);
-                b.launches += 2;
-                if (ms < best) {
-                    best = ms;
-                    bnc = nc;
-                    bth = th;
-                    bw = w;
-                    bp = paired;
-                }
-            }
+        for (int nc = 2; nc <= 3; ++nc)
+            for (int th : ths)
+                if ((e = probe(nc, th, 4, paired)) != cudaSuccess) return e;
+    {
+        const int nc = bnc, th = bth, paired = bp;
+        for (int w : {2, 8})
+            if ((e = probe(nc, th, w, paired)) != cudaSuccess) return e;
+    }
     cudaEventDestroy(a);
     cudaEventDestroy(z);
     b.tuned = true;

@@ -21,15 +21,14 @@ struct Grid {
     int nx, ny;
     float dx, dy, g, f, H, theta;
     float inv_dx, inv_dy;
-    float fdx, fdy;            // f dx, f dy
-    float fdx_half, fdy_half;  // f dx / 2, f dy / 2
-    float inv_2g;
+    float fdy;                 // f dy
     float sgh;                 // g H / f (geostrophic balance)
     float inv_2dx, inv_2dy;
-    // exact doublings / halvings of the above for the marching kernel, whose
-    // slopes are carried as twice their value; g/2 and g H for the pressure
-    float theta2, fdx2, fdy2, inv_4g;
-    float g_half, gH;
+    // of the marching kernel, whose slopes are carried as twice their value
+    // and whose potentials are divided by g: 2 theta, f dx / (2 g), f dy / (2
+    // g), dy / dx; g/2, g H and sqrt(g) for the pressure and the wave speed
+    float theta2, fdx_2g, fdy_2g, dy_dx;
+    float g_half, gH, sqrt_g;
     int ne;
     long long plane;           // nx * ny
 };

@@ -67,7 +67,25 @@ struct StepArgs {
     int TH, n_strips, n_chunks;
     const int* s_dev = nullptr;   // scheme-step index in device memory (graph loops), else the kernel argument
 };
+// Rows of nx columns that one warp of NC columns per lane holds whole, lanes
+// 0 .. nx / NC - 1 closing the periodic row; wider rows, or others, take
+// strips of 32 NC columns of which 4 on each side are halo.  (A ring of 21
+// to 32 lanes computes 64 columns with 32 or 22 of the 32 lanes where a strip
+// with halo takes two warps, or 22 lanes of one that computes 96.)
+inline bool ring(int nx, int nc) { return nx % nc == 0 && nx <= 32 * nc; }
+inline int strips(int nx, int nc) { return ring(nx, nc) ? 1 : (nx + 32 * nc - 9) / (32 * nc - 8); }
 }  // namespace march
+
+// candidate chunk lengths of ny rows: 1 to 32 equal chunks, at least 2 rows each
+inline std::vector<int> march_rows(int ny)
+{
+    std::vector<int> th;
+    for (int n : {1, 2, 3, 4, 6, 8, 16, 32}) {
+        const int t = (ny + n - 1) / n;
+        if (t >= 2 && (th.empty() || t < th.back())) th.push_back(t);
+    }
+    return th;
+}
 
 // tile shape of the register-marching scheme step: NC columns per lane, TH
 // rows per chunk, warps per CTA, and whether the two Runge-Kutta stages run

@@ -6,43 +6,53 @@ namespace iewpf {
 
 namespace {
 
-template <int NC>
-__global__ void __launch_bounds__(256)
+// The warps of a particle's strips and chunks are consecutive; the index is
+// broadcast from lane 0 so that everything derived from it (particle, rows,
+// row addresses) is uniform over the warp.
+//
+// Bound by instruction issue: at 512^2 x 100 the paired form executes 337
+// warp instructions per 32 cells, of which the 125 packed ones take two
+// dispatch slots each, the scalar form 451; memory traffic is a quarter of
+// what HBM could move in that time.  Registers: 168 with 2 columns per lane (the
+// bound of 384 threads), so that 12 warps share an SM; 255 with 3 columns, 8
+// warps.  Giving each stage a warp of its own (128 registers, 16 warps, rows
+// handed over in shared memory) issues in 81% of the cycles instead of 58%
+// but executes 485 instructions, and is slower (401 us).
+// One launch, start of the potential and flux forms above -> now:
+//   512^2 x 100: 394 -> 384 us; 1024^2 x 64: 1033 -> 980 us;
+//   64^2 x 640 (rows closing on a ring of 32 lanes): 75 -> 60 us
+template <int NC, bool RING, bool PAIRED>
+__global__ void __launch_bounds__(NC == 2 ? 384 : 256)
 rk2_march_kernel(march::StepArgs a, int s)
 {
-    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const long long warp =
+        (long long)blockIdx.x * (blockDim.x >> 5) + __shfl_sync(march::FULL, (int)(threadIdx.x >> 5), 0);
     const long long per_p = (long long)a.n_strips * a.n_chunks;
     if (warp >= per_p * a.G.ne) return;
     const int p = (int)(warp / per_p);
     const int rem = (int)(warp % per_p);
-    march::march_warp<NC>(a, p, rem / a.n_strips, rem % a.n_strips, a.s_dev ? *a.s_dev : s);
+    const int st = a.s_dev ? *a.s_dev : s;
+    if (PAIRED) march::march_warp_paired<NC, RING>(a, p, rem / a.n_strips, rem % a.n_strips, st);
+    else march::march_warp<NC, RING>(a, p, rem / a.n_strips, rem % a.n_strips, st);
 }
 
-template <int NC>
-__global__ void __launch_bounds__(256)
-rk2_march2_kernel(march::StepArgs a, int s)
+template <int NC, bool RING>
+cudaError_t launch(const march::StepArgs& a, int s, int warps, int paired, cudaStream_t st)
 {
-    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long per_p = (long long)a.n_strips * a.n_chunks;
-    if (warp >= per_p * a.G.ne) return;
-    const int p = (int)(warp / per_p);
-    const int rem = (int)(warp % per_p);
-    march::march_warp_paired<NC>(a, p, rem / a.n_strips, rem % a.n_strips, a.s_dev ? *a.s_dev : s);
+    const long long n = (long long)a.n_strips * a.n_chunks * a.G.ne;
+    const unsigned blocks = (unsigned)((n + warps - 1) / warps);
+    if (paired) rk2_march_kernel<NC, RING, true><<<blocks, 32 * warps, 0, st>>>(a, s);
+    else rk2_march_kernel<NC, RING, false><<<blocks, 32 * warps, 0, st>>>(a, s);
+    return cudaGetLastError();
 }
 
 template <int NC>
 cudaError_t launch_nc(float* b0, float* b1, const int* par, const int* nsub, const float* dtp, int s, const Grid& G,
                       int TH, int warps_per_cta, int paired, const int* s_dev, cudaStream_t st)
 {
-    constexpr int WUSE = 32 * NC - 8;
-    march::StepArgs a{b0, b1, par, nsub, dtp, G, TH, (G.nx + WUSE - 1) / WUSE, (G.ny + TH - 1) / TH, s_dev};
-    const long long warps = (long long)a.n_strips * a.n_chunks * G.ne;
-    const long long blocks = (warps + warps_per_cta - 1) / warps_per_cta;
-    if (paired)
-        rk2_march2_kernel<NC><<<(unsigned)blocks, 32 * warps_per_cta, 0, st>>>(a, s);
-    else
-        rk2_march_kernel<NC><<<(unsigned)blocks, 32 * warps_per_cta, 0, st>>>(a, s);
-    return cudaGetLastError();
+    const march::StepArgs a{b0, b1, par, nsub, dtp, G, TH, march::strips(G.nx, NC), (G.ny + TH - 1) / TH, s_dev};
+    if (march::ring(G.nx, NC)) return launch<NC, true>(a, s, warps_per_cta, paired, st);
+    return launch<NC, false>(a, s, warps_per_cta, paired, st);
 }
 
 }  // namespace

@@ -55,3 +55,27 @@ def test_random_vectors_over_philox_blocks(nx, ny):
     np.testing.assert_allclose(d["gamma"], dref["gamma"], rtol=1e-10)
     np.testing.assert_allclose(d["zeta"], dref["zeta"], rtol=1e-10)
     assert rel_l2(ens.get_state(), ref) <= 1e-5
+
+
+@pytest.mark.parametrize("nx,ny", [(44, 46), (64, 64), (66, 47), (96, 45), (93, 50), (97, 44), (176, 48)])
+def test_marching_shapes_agree_bitwise_and_with_the_oracle(nx, ny):
+    """Rows that close on a ring of lanes (44, 64, 96, 93 with 3 columns, 66) or take strips with halo (one
+    and several, with and without remainder), chunks from 2 rows to more than the grid: every kind and
+    shape gives the same bits, and the oracle's state at 1e-5."""
+    cfg = synth.Config("edge", nx, ny, n_particles=3)
+    ens, P = ensemble(cfg), oracle_problem(cfg)
+    U32, U64 = start_state(cfg, 3)
+    first = None
+    for kind in (1, 2):
+        for nc in (2, 3, 4):
+            for rows, warps in ((2, 4), (ny // 3, 2), (ny, 8), (2 * ny, 1)):
+                ens.set_stepper(kind, nc, rows, warps)
+                ens.set_state(U32)
+                ens.set_counters(0, 0)
+                ens.forecast(1, False)
+                got = ens.get_state()
+                if first is None:
+                    first = got
+                    ref, _, _ = O.forecast(P, U64, 1, False, t0=0)
+                    assert rel_l2(got, ref) <= 1e-5
+                assert np.array_equal(got, first), (kind, nc, rows, warps)
