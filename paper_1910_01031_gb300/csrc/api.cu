@@ -828,7 +828,11 @@ int iewpf_create(const iewpf_params_t* params, const double* mooring_xy, iewpf_c
     if ((rc = dalloc(ctx, &ctx->d_s, 1)) || (rc = dalloc(ctx, &ctx->d_step, 1)) || (rc = dalloc(ctx, &ctx->d_iters, 1)))
         return bail(rc);
     if (cudaStreamCreateWithFlags(&ctx->st2, cudaStreamNonBlocking) != cudaSuccess) return bail(IEWPF_ECUDA);
-    std::vector<float> K32(ctx->K64.begin(), ctx->K64.end());
+    // [2R+1][2R+1][2 x 3]: the six values at an offset together (pull_row)
+    const size_t KW = (size_t)(2 * ctx->R + 1) * (2 * ctx->R + 1);
+    std::vector<float> K32(6 * KW);
+    for (size_t o = 0; o < KW; ++o)
+        for (int k = 0; k < 6; ++k) K32[6 * o + k] = (float)ctx->K64[k * KW + o];
     std::vector<float> M32(ctx->M49.begin(), ctx->M49.end());
     if (cudaMemsetAsync(ctx->buf[0], 0, state * sizeof(float), ctx->st) != cudaSuccess ||
         cudaMemsetAsync(ctx->buf[1], 0, state * sizeof(float), ctx->st) != cudaSuccess ||

@@ -20,6 +20,7 @@
 #include "batch.h"
 #include "march_dev.cuh"
 #include "qhalf_dev.cuh"
+#include "tc_dev.cuh"
 
 namespace iewpf {
 
@@ -30,7 +31,7 @@ enum Space : int {
     SP_PART = 0,   // particles
     SP_CFL,        // CFL slices: particle x slice of the plane
     SP_STEP,       // scheme-step warps: particle x chunk x strip
-    SP_TILE,       // fine tiles: particle x tile
+    SP_TILE,       // fine tiles: group of particles (BatchImpl::fine_parts) x tile
     SP_OBS,        // observations
     SP_BIN,        // tiles of the observation lists (one per problem tile)
     SP_INN,        // particle x observation
@@ -38,7 +39,6 @@ enum Space : int {
     SP_DOT,        // dot-product slices: particle x slice
     SP_FR,         // particle x coarse point
     SP_NRM,        // particle x Philox block of the coarse normals and of the posterior field
-    SP_FTILE,      // model-error fine tiles (FINE_TX x FINE_TY): particle x tile
     SP_COUNT
 };
 
@@ -192,18 +192,20 @@ __global__ void b_soar(BatchDev B)
     }
 }
 
-template <bool PULL>
-__global__ void __launch_bounds__(NTHREADS) b_fine(BatchDev B)
+template <bool PULL, int PB, int SUB>
+__global__ void __launch_bounds__(NTHREADS, PB <= 4 ? 2 : 1) b_fine(BatchDev B)
 {
     constexpr int TX = qhalf::FINE_TX, TY = qhalf::FINE_TY;
-    const long long* pre = space(B, PULL ? SP_TILE : SP_FTILE);
+    constexpr int PARTS = qhalf::fine_parts(PB, SUB);
+    extern __shared__ __align__(16) float fine_smem[];
+    const long long* pre = space(B, SP_TILE);
     for (long long q = blockIdx.x; q < pre[B.n]; q += gridDim.x) {
         const int i = find_inst(pre, B.n, q);
         const BInst& I = B.inst[i];
-        const int ntx = (I.G.nx + TX - 1) / TX, nty = (I.G.ny + TY - 1) / TY;
+        const int tiles = ((I.G.nx + TX - 1) / TX) * ((I.G.ny + TY - 1) / TY);
         const long long r = q - pre[i];
-        const int p = (int)(r / (ntx * nty));
-        const int tile = (int)(r % (ntx * nty));
+        const int p0 = (int)(r / tiles) * PARTS;
+        const int tile = (int)(r % tiles);
         QhalfArgs A{};
         A.b0 = I.step.buf0;
         A.b1 = I.step.buf1;
@@ -222,8 +224,7 @@ __global__ void __launch_bounds__(NTHREADS) b_fine(BatchDev B)
         }
         const Grid G = I.G;
         const Coarse C = I.C;
-        qhalf::fine_tile<PULL, TX, TY>(A, G, C, (tile % ntx) * TX, (tile / ntx) * TY, p, tile,
-                                       I.soar + (long long)p * I.NR);
+        qhalf::fine_cta<PULL, PB, SUB>(A, G, C, tile, p0, I.soar, fine_smem, PULL ? MAX_TILE_OBS : 0, false);
     }
 }
 
@@ -374,12 +375,12 @@ __global__ void b_pack_diag(BatchDev B, double* out)
     }
 }
 
-int resident_blocks(const void* fn, int threads)
+int resident_blocks(const void* fn, int threads, size_t smem = 0)
 {
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads, smem);
     return std::max(1, sms * std::max(1, per));
 }
 
@@ -414,6 +415,7 @@ struct BatchImpl {
     bool fgraph_err = false;
     int nc = 2;
     int warps = 4;
+    int fine_parts = 1; // particles per CTA of the fine stage (qhalf::fine_choice)
     bool ring = false;  // every row held by one ring of lanes (march::ring)
     int paired = 0;     // scheme step with the two stages in f32x2 pairs (nc 2 or 3)
     int fixed = 0;
@@ -456,6 +458,21 @@ int grid_for(K kern, int threads, long long work_items_per_block_units)
     return (int)std::max<long long>(1, std::min<long long>(cap, work_items_per_block_units));
 }
 
+template <bool PULL>
+cudaError_t launch_fine(BatchImpl& b, cudaStream_t st)
+{
+    auto run = [&](auto kern, int parts) -> cudaError_t {
+        // the lists of the pull in dynamic shared memory (at most 34 KB)
+        const size_t smem = PULL ? qhalf::fine_list_bytes(MAX_TILE_OBS, parts) : 0;
+        const int g = (int)std::min<long long>(items(b, SP_TILE), resident_blocks((const void*)kern, NTHREADS, smem));
+        kern<<<std::max(1, g), NTHREADS, smem, st>>>(dev_view(b));
+        return cudaGetLastError();
+    };
+    if (b.fine_parts == qhalf::fine_parts(4, 1)) return run(b_fine<PULL, 4, 1>, b.fine_parts);
+    if (b.fine_parts == qhalf::fine_parts(4, 4)) return run(b_fine<PULL, 4, 4>, b.fine_parts);
+    return run(b_fine<PULL, 1, 4>, b.fine_parts);
+}
+
 }  // namespace
 
 cudaError_t batch_set_step_shape(BatchImpl& b, int nc, int th, int warps, int paired)
@@ -494,16 +511,21 @@ cudaError_t batch_init(BatchImpl& b, const std::vector<BInst>& insts)
     b.pre.assign((size_t)SP_COUNT * (b.n + 1), 0);
     long long acc[SP_COUNT] = {0};
     b.obs_off.assign(b.n + 1, 0);
+    b.fine_parts = qhalf::fine_choice(
+        [&](int n) {
+            long long t = 0;
+            for (const BInst& I : insts)
+                t += (long long)((I.G.nx + OBS_TX - 1) / OBS_TX) * ((I.G.ny + OBS_TY - 1) / OBS_TY) * ((I.G.ne + n - 1) / n);
+            return t;
+        },
+        tc::sm_count());
     for (int i = 0; i < b.n; ++i) {
         const BInst& I = insts[i];
         const long long ne = I.G.ne;
         const long long slices = (I.G.plane + kCflSlice - 1) / kCflSlice;
         const long long tiles = (long long)((I.G.nx + OBS_TX - 1) / OBS_TX) * ((I.G.ny + OBS_TY - 1) / OBS_TY);
-        const long long ftiles = (long long)((I.G.nx + qhalf::FINE_TX - 1) / qhalf::FINE_TX) *
-                                 ((I.G.ny + qhalf::FINE_TY - 1) / qhalf::FINE_TY);
-        const long long cnt[SP_COUNT] = {ne, ne * slices, 0, ne * tiles, I.nobs, tiles, ne * I.nobs,
-                                         4LL * I.nobs * I.nobs, ne * I.nblk, ne * I.NR, ne * ((I.NR + 3) / 4),
-                                         ne * ftiles};
+        const long long cnt[SP_COUNT] = {ne, ne * slices, 0, (ne + b.fine_parts - 1) / b.fine_parts * tiles, I.nobs, tiles, ne * I.nobs,
+                                         4LL * I.nobs * I.nobs, ne * I.nblk, ne * I.NR, ne * ((I.NR + 3) / 4)};
         for (int sp = 0; sp < SP_COUNT; ++sp) {
             b.pre[(size_t)sp * (b.n + 1) + i] = acc[sp];
             acc[sp] += cnt[sp];
@@ -612,7 +634,7 @@ static cudaError_t capture_model_step(BatchImpl& b, cudaStream_t st, cudaStream_
         b.launches += 1;
         b_normals<<<grid_for(b_normals, 256, (items(b, SP_NRM) + 255) / 256), 256, 0, st>>>(B);
         b_soar<false><<<grid_for(b_soar<false>, 256, (items(b, SP_FR) + 255) / 256), 256, 0, st>>>(B);
-        b_fine<false><<<grid_for(b_fine<false>, NTHREADS, items(b, SP_FTILE)), NTHREADS, 0, st>>>(B);
+        if ((e = launch_fine<false>(b, st)) != cudaSuccess) return e;
         b.launches += 3;
     }
     b_count<<<(b.n + 127) / 128, 128, 0, st>>>(B, 0);
@@ -638,7 +660,7 @@ static cudaError_t capture_analysis(BatchImpl& b, cudaStream_t st)
     b_form_r<<<grid_for(b_form_r, 256, (items(b, SP_NRM) + 255) / 256), 256, 0, st>>>(B);
     b_block_seq<<<grid_for(b_block_seq, 64, items(b, SP_PART)), 64, 0, st>>>(B);
     b_soar<true><<<grid_for(b_soar<true>, 256, (items(b, SP_FR) + 255) / 256), 256, 0, st>>>(B);
-    b_fine<true><<<grid_for(b_fine<true>, NTHREADS, items(b, SP_TILE)), NTHREADS, 0, st>>>(B);
+    if ((e = launch_fine<true>(b, st)) != cudaSuccess) return e;
     b_count<<<(b.n + 127) / 128, 128, 0, st>>>(B, 1);
     b_nonfinite<<<grid_for(b_nonfinite, NTHREADS, items(b, SP_CFL)), NTHREADS, 0, st>>>(B);
     b_pack_diag<<<(b.n + 127) / 128, 128, 0, st>>>(B, b.d_diag);

@@ -115,7 +115,7 @@ struct QhalfArgs {
     const float* x;           // [ne][N_R]
     // optimal-proposal pull (may be disabled)
     int with_pull;
-    const float* K;           // [2][3][2R+1][2R+1]
+    const float* K;           // [2R+1][2R+1][2][3]: the stencil values at an offset together
     int R;
     const int* obs_cell;      // [nobs][2]
     const double* Sd;         // [ne][2 nobs]

@@ -1,6 +1,10 @@
 // Model error and analysis update (Sec. 3.2 and 4.6 of arXiv 1910.01031),
 // one problem per launch; the device code is in qhalf_dev.cuh.
+#include <algorithm>
+#include <type_traits>
+
 #include "qhalf_dev.cuh"
+#include "tc_dev.cuh"
 
 namespace iewpf {
 
@@ -33,14 +37,33 @@ __global__ void coarse_soar_kernel(const float* __restrict__ src, const float* _
 using qhalf::FINE_TX;
 using qhalf::FINE_TY;
 
-template <bool PULL>
-__global__ void __launch_bounds__(NTHREADS)
-qhalf_fine_kernel(QhalfArgs A, Grid G, Coarse C)
+template <bool PULL, int PB, int SUB>
+__global__ void __launch_bounds__(NTHREADS, PB <= 4 ? 2 : 1)
+qhalf_fine_kernel(QhalfArgs A, Grid G, Coarse C, int cap, int k_in_smem)
 {
-    const long long NR = (long long)C.nRx * C.nRy;
-    constexpr int TX = FINE_TX, TY = FINE_TY;
-    qhalf::fine_tile<PULL, TX, TY>(A, G, C, blockIdx.x * TX, blockIdx.y * TY, blockIdx.z,
-                                   blockIdx.y * gridDim.x + blockIdx.x, A.soar_buf + (long long)blockIdx.z * NR);
+    extern __shared__ __align__(16) float fine_smem[];
+    qhalf::fine_cta<PULL, PB, SUB>(A, G, C, blockIdx.x, blockIdx.y * qhalf::fine_parts(PB, SUB), A.soar_buf, fine_smem,
+                                   cap, k_in_smem);
+}
+
+constexpr size_t kStencilSmem = 64 * 1024;      // c_Omega up to 3 (44 KB)
+
+template <bool PULL, int PB, int SUB>
+cudaError_t launch_fine(const QhalfArgs& A, const Grid& G, const Coarse& C, int tiles, cudaStream_t st)
+{
+    constexpr int parts = qhalf::fine_parts(PB, SUB);
+    const int cap = PULL ? std::min(A.nobs, MAX_TILE_OBS) : 0;
+    const size_t kbytes = PULL && PB > 1 ? 6 * sizeof(float) * (2 * A.R + 1) * (2 * A.R + 1) : 0;
+    const int k_in_smem = kbytes > 0 && kbytes <= kStencilSmem;
+    const size_t smem = qhalf::fine_list_bytes(cap, parts) + (k_in_smem ? kbytes : 0);
+    if (PULL) {
+        const cudaError_t e = tc::smem_attr_once<qhalf_fine_kernel<PULL, PB, SUB>>(
+            (int)(qhalf::fine_list_bytes(MAX_TILE_OBS, parts) + kStencilSmem));
+        if (e != cudaSuccess) return e;
+    }
+    qhalf_fine_kernel<PULL, PB, SUB>
+        <<<dim3((unsigned)tiles, (unsigned)((G.ne + parts - 1) / parts)), NTHREADS, smem, st>>>(A, G, C, cap, k_in_smem);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -62,10 +85,16 @@ cudaError_t launch_qhalf(const QhalfArgs& A, const Grid& G, const Coarse& C, cud
         src = A.xi_buf;
     }
     coarse_soar_kernel<<<dim3((unsigned)((NR + 255) / 256), G.ne), 256, 0, st>>>(src, A.wtab, G, C, A.soar_buf);
-    const dim3 grid((G.nx + FINE_TX - 1) / FINE_TX, (G.ny + FINE_TY - 1) / FINE_TY, G.ne);
-    if (A.with_pull) qhalf_fine_kernel<true><<<grid, NTHREADS, 0, st>>>(A, G, C);
-    else qhalf_fine_kernel<false><<<grid, NTHREADS, 0, st>>>(A, G, C);
-    return cudaGetLastError();
+    const int tiles = ((G.nx + FINE_TX - 1) / FINE_TX) * ((G.ny + FINE_TY - 1) / FINE_TY);
+    const int parts = qhalf::fine_choice(
+        [&](int n) { return (long long)tiles * ((G.ne + n - 1) / n); }, tc::sm_count());
+    auto run = [&](auto pull) {
+        constexpr bool P = decltype(pull)::value;
+        if (parts == qhalf::fine_parts(4, 1)) return launch_fine<P, 4, 1>(A, G, C, tiles, st);
+        if (parts == qhalf::fine_parts(4, 4)) return launch_fine<P, 4, 4>(A, G, C, tiles, st);
+        return launch_fine<P, 1, 4>(A, G, C, tiles, st);
+    };
+    return A.with_pull ? run(std::true_type{}) : run(std::false_type{});
 }
 
 }  // namespace iewpf

@@ -4,7 +4,7 @@
 //   Philox normals once per coarse point (normals_block)
 //   -> 5x5 SOAR once per coarse point (soar_point)
 //   -> per fine tile: bicubic to the tile + 1-cell ring, central-difference
-//      geostrophic momentum, read-modify-write of the state (fine_tile).
+//      geostrophic momentum, read-modify-write of the state (fine_cta).
 // The analysis update reuses the fine stage with the posterior coarse field
 // and adds the optimal-proposal pull (eq. detailedOPDUpdate) in the same
 // read-modify-write.
@@ -19,29 +19,6 @@ constexpr int TAB_MAX = 45;                   // 3 c for c <= 15
 // fine tiles of the model error and of the analysis update (the tiles the
 // observation lists are binned by)
 constexpr int FINE_TX = OBS_TX, FINE_TY = OBS_TY;
-
-// Per observation of a tile's list, once per tile: the minimum-image offset
-// of the tile origin (x0, y0) from the observed cell, in (-n/2, n/2], and the
-// particle's S d as float; the cells of the tile then add their own offset
-// (at most one period above).  Returns the list length.  Ends with a barrier.
-__device__ __forceinline__ int tile_obs_prep(const QhalfArgs& A, const Grid& G, int x0, int y0, int p, int tile,
-                                             int* ox0, int* oy0, float* su, float* sv)
-{
-    const int n = min(A.tile_cnt[tile], MAX_TILE_OBS);
-    for (int q = threadIdx.x; q < n; q += NTHREADS) {
-        const int l = A.tile_obs[tile * A.tile_cap + q];
-        int ox = pmod(x0 - A.obs_cell[2 * l], G.nx);
-        int oy = pmod(y0 - A.obs_cell[2 * l + 1], G.ny);
-        if (ox > G.nx / 2) ox -= G.nx;
-        if (oy > G.ny / 2) oy -= G.ny;
-        ox0[q] = ox;
-        oy0[q] = oy;
-        su[q] = (float)A.Sd[(long long)p * 2 * A.nobs + 2 * l];
-        sv[q] = (float)A.Sd[(long long)p * 2 * A.nobs + 2 * l + 1];
-    }
-    __syncthreads();
-    return n;
-}
 
 // Coarse stages once per coarse point.  Normals of block q (counter q) of a
 // Philox stream: words (0, 1) and (2, 3) give the Box-Muller pairs of normals
@@ -95,212 +72,341 @@ __device__ __forceinline__ float soar_point(const float* __restrict__ src, const
     return acc;
 }
 
-// One fine tile (TX x TY cells) from the SOAR field so_g [N_R] of particle
-// p: bicubic to the tile and its 1-cell ring, geostrophic momentum, optional
-// pull (`tile` indexes the observation lists, binned by the same tiles), and
-// the read-modify-write of the state.  The interpolation runs separably (rows
-// first).  Called by whole CTAs of NTHREADS threads; a CTA may call it for
-// several tiles in turn.
-template <bool PULL, int TX, int TY>
-__device__ __forceinline__ void fine_tile(const QhalfArgs& A, const Grid& G, const Coarse& C, int x0, int y0, int p,
-                                          int tile, const float* __restrict__ so_g)
+// The fine stage: a warp marches down a strip of 32 columns of PB particles
+// at once, one column per lane, with no shared memory between lanes and no
+// barriers: the four coarse rows around the current row, interpolated in x at
+// the lane's column, roll in registers (a new one every c rows), the
+// y-interpolation gives the field of one row, three rows of it roll for the
+// y-difference, and the x-difference takes the neighbours' values by shuffle.
+// The two columns beside the strip, which only that difference needs, are one
+// more column per warp: lanes 2 pp and 2 pp + 1 carry those of particle pp.
+// A coarse row is one load per particle (lane l the l-th coarse column the
+// strip touches, requested an interval ahead) and four shuffles, where the
+// strip's coarse columns fit the lanes (c >= 2), else four loads.
+// PB particles share the row's weights and, with the pull, each load of the
+// stencil: those loads bound the pull when every particle makes its own.
+//
+// Pull: each listed observation that reaches the row of the strip, in list
+// order, adds its six stencil products to the cells it reaches (offset within
+// R of the cell in the minimum image, both axes: the stencil's reach 2R + 1
+// lies within the grid, iewpf_create refuses smaller ones, so each cell sees
+// one image).  The sum of a cell starts from the interpolated field and its
+// balanced momentum; the state is rewritten once.
+//
+// The CTA: TY rows x two strips (the OBS_TX x OBS_TY tiles of the observation
+// lists) of fine_parts(PB, SUB) particles; four warps per strip take a group of PB
+// particles each (SUB = 1), or a quarter of the rows of one group (SUB = 4, for
+// ensembles too small to fill the GPU otherwise).
+//
+// Bound by latency and issue with 4 particles per warp (128 registers, 16 warps
+// per SM); 8 per warp halve the stencil's loads again but also the warps.
+// Analysis update: the tile kernel it replaced interpolated through shared
+// memory with four barriers and then applied one observation at a time to the
+// whole tile, each particle loading the stencil anew and a barrier between
+// observations: 11.1 ms at 624^2 x 1000 (7 of 1521 observations reach a
+// cell), now 4.1 ms; 4.2 -> 2.0 ms at 1024^2 x 256 (2.7 of 1521); 234 -> 180 us
+// at 512^2 x 100 (64 drifters).  Model error: 168 -> 153 us at 512^2 x 100, 48
+// -> 38 us at 256^2 x 100.
+constexpr int STRIPS = OBS_TX / 32;
+constexpr int GROUPS = NTHREADS / 32 / STRIPS;
+__host__ __device__ constexpr int fine_parts(int PB, int SUB) { return PB * (GROUPS / SUB); }
+// host: (PB, SUB) by the number of particles in a CTA, as many as leave every
+// SM a CTA: 16 (4, 1), 4 (4, 4) or 1 (1, 4); ctas(parts) counts the CTAs
+template <class F>
+inline int fine_choice(F ctas, int sms)
 {
-    constexpr int FW = TX + 2, FH = TY + 2, SXW = FW + 3, SXH = FH + 3;
-    static_assert(!PULL || (TX == OBS_TX && TY == OBS_TY), "pull tiles follow the observation lists");
-    // the coarse patch, its rows interpolated and the interpolated field share
-    // one pool; with the pull, the tile's per-cell sums take its start once
-    // the interpolated field has been read
-    constexpr int SO_N = SXH * SXW, ROWS_N = SXH * FW, DETA_N = FH * FW;
-    static_assert(SO_N + ROWS_N + DETA_N >= 3 * TX * TY, "pull sums fit the pool");
-    __shared__ float pool[SO_N + ROWS_N + DETA_N];
-    float(*so)[SXW] = reinterpret_cast<float(*)[SXW]>(pool);
-    float(*rows)[FW] = reinterpret_cast<float(*)[FW]>(pool + SO_N);
-    float(*deta)[FW] = reinterpret_cast<float(*)[FW]>(pool + SO_N + ROWS_N);
-    __shared__ int colA[FW], rowB[FH];
-    __shared__ float colW[FW][4], rowW[FH][4];
+    for (int parts : {fine_parts(4, 1), fine_parts(4, 4)})
+        if (ctas(parts) >= sms) return parts;
+    return fine_parts(1, 4);
+}
 
-    const int tid = threadIdx.x;
-    __syncthreads();   // the shared arrays may still be in use by the previous tile
-    float tdum;
-    const int a_lo = coarse_interval(x0 - 1, C.nRx, C.c, C.o, G.nx, tdum);
-    const int a_hi = coarse_interval(x0 + TX, C.nRx, C.c, C.o, G.nx, tdum);
-    const int b_lo = coarse_interval(y0 - 1, C.nRy, C.c, C.o, G.ny, tdum);
-    const int b_hi = coarse_interval(y0 + TY, C.nRy, C.c, C.o, G.ny, tdum);
-    const int nsx = a_hi - a_lo + 4, nsy = b_hi - b_lo + 4;     // SOAR, first at a_lo - 1
-    for (int i = tid; i < FW; i += NTHREADS) {
-        float t;
-        const int a = coarse_interval(x0 - 1 + i, C.nRx, C.c, C.o, G.nx, t);
-        colA[i] = a - a_lo;
-        cubic_weights(t, colW[i]);
-    }
-    for (int i = tid; i < FH; i += NTHREADS) {
-        float t;
-        const int b = coarse_interval(y0 - 1 + i, C.nRy, C.c, C.o, G.ny, t);
-        rowB[i] = b - b_lo;
-        cubic_weights(t, rowW[i]);
-    }
-    // the coarse patch, a row per warp (the indices lie within a period or
-    // two of the grid: wrapped by steps, not by an integer modulo)
-    for (int sy = tid >> 5; sy < nsy; sy += NTHREADS / 32) {
-        int r = b_lo - 1 + sy;
-        while (r < 0) r += C.nRy;
-        while (r >= C.nRy) r -= C.nRy;
-        for (int sx = tid & 31; sx < nsx; sx += 32) {
-            int c = a_lo - 1 + sx;
-            while (c < 0) c += C.nRx;
-            while (c >= C.nRx) c -= C.nRx;
-            so[sy][sx] = so_g[r * C.nRx + c];
-        }
-    }
-    __syncthreads();
-    // rows: the x-interpolation of every SOAR row at every fine column; a
-    // lane keeps its columns' taps and weights, the warps take the rows
-    {
-        const int lane = tid & 31, warp = tid >> 5;
+// Dynamic shared memory of one CTA (16-byte aligned) for lists of up to cap
+// observations of `parts` particles: S d as (su, su', sv, sv') of each pair of
+// particles, the pairs of an observation together ((su, sv) of a single
+// particle), then the observations' offsets from the tile origin, then the
+// copy of the stencil.
+__host__ __device__ constexpr size_t fine_list_bytes(int cap, int parts) { return (size_t)cap * (8 + 8 * (size_t)parts); }
+
+struct FineRows {
+    float4 w[FINE_TY + 2];      // y-weights of rows y0 - 1 .. y0 + TY
+    int b[FINE_TY + 2];         // and their coarse intervals
+};
+
+__device__ __forceinline__ void column_taps(int x, const Grid& G, const Coarse& C, int& a, float w[4])
+{
+    float t;
+    a = coarse_interval(x, C.nRx, C.c, C.o, G.nx, t);
+    cubic_weights(t, w);
+}
+
+__device__ __forceinline__ float taps(const float w[4], float v0, float v1, float v2, float v3)
+{
+    float v = 0.0f;
+    v = fmaf(w[0], v0, v);
+    v = fmaf(w[1], v1, v);
+    v = fmaf(w[2], v2, v);
+    v = fmaf(w[3], v3, v);
+    return v;
+}
+
+// adds (su, sv) of the warp's PB particles times the stencil values k[6] (su:
+// 0..2, sv: 3..5) to their sums; pairs of particles in packed FMAs (each half
+// rounds as the scalar instruction)
+template <int PB>
+__device__ __forceinline__ void pull_add(float (&acc)[3][PB], const float* __restrict__ s, const float k[6])
+{
+    if constexpr (PB == 1) {
+        const float2 v = *reinterpret_cast<const float2*>(s);
 #pragma unroll
-        for (int j = 0; j < (FW + 31) / 32; ++j) {
-            const int fx = lane + 32 * j;
-            if (fx < FW) {
-                const int a = colA[fx];
-                const float w0 = colW[fx][0], w1 = colW[fx][1], w2 = colW[fx][2], w3 = colW[fx][3];
-                for (int sy = warp; sy < nsy; sy += NTHREADS / 32) {
-                    float row = 0.0f;
-                    row = fmaf(w0, so[sy][a], row);
-                    row = fmaf(w1, so[sy][a + 1], row);
-                    row = fmaf(w2, so[sy][a + 2], row);
-                    row = fmaf(w3, so[sy][a + 3], row);
-                    rows[sy][fx] = row;
-                }
+        for (int f = 0; f < 3; ++f) acc[f][0] = fmaf(v.y, k[3 + f], fmaf(v.x, k[f], acc[f][0]));
+    } else {
+#pragma unroll
+        for (int pp = 0; pp < PB; pp += 2) {
+            const float4 v = *reinterpret_cast<const float4*>(s + 2 * pp);
+#pragma unroll
+            for (int f = 0; f < 3; ++f) {
+                float2 a = make_float2(acc[f][pp], acc[f][pp + 1]);
+                a = __ffma2_rn(make_float2(v.x, v.y), make_float2(k[f], k[f]), a);
+                a = __ffma2_rn(make_float2(v.z, v.w), make_float2(k[3 + f], k[3 + f]), a);
+                acc[f][pp] = a.x;
+                acc[f][pp + 1] = a.y;
             }
         }
     }
-    __syncthreads();
-    // the y-interpolation: a row of the tile per warp, the lanes along it
-    for (int fy = tid >> 5; fy < FH; fy += NTHREADS / 32) {
-        const int b = rowB[fy];
-        const float w0 = rowW[fy][0], w1 = rowW[fy][1], w2 = rowW[fy][2], w3 = rowW[fy][3];
-        for (int fx = tid & 31; fx < FW; fx += 32) {
-            float acc = 0.0f;
-            acc = fmaf(w0, rows[b][fx], acc);
-            acc = fmaf(w1, rows[b + 1][fx], acc);
-            acc = fmaf(w2, rows[b + 2][fx], acc);
-            acc = fmaf(w3, rows[b + 3][fx], acc);
-            deta[fy][fx] = acc;
+}
+
+// the pull of one row: ty, sx the row and the strip's first column in the
+// tile; sd the warp's S d of observation 0, sd_stride floats per observation;
+// K [2R+1][2R+1][6]
+template <int PB>
+__device__ __forceinline__ void pull_row(float (&acc)[3][PB], const Grid& G, int R, const int2* __restrict__ off,
+                                         int n_obs, const float* __restrict__ sd, int sd_stride,
+                                         const float* __restrict__ K, int ty, int sx)
+{
+    const int lane = threadIdx.x & 31, W = 2 * R + 1;
+    for (int q0 = 0; q0 < n_obs; q0 += 32) {
+        // lane j: does observation q0 + j reach a cell of this row, at which
+        // stencil row (element kb) and, for the strip's first column, at which
+        // column xo (0 .. 2R, or a period above)
+        bool in = false;
+        int kb = 0, xo = 0;
+        if (q0 + lane < n_obs) {
+            const int2 o = off[q0 + lane];
+            int oy = o.y + ty;
+            const int ox = o.x + sx;
+            if (oy > R) oy -= G.ny;
+            in = oy >= -R && oy <= R && ((ox <= R && ox + 31 >= -R) || (ox - G.nx <= R && ox + 31 - G.nx >= -R));
+            kb = (oy + R) * W * 6;
+            xo = ox + R;
+        }
+        for (unsigned mask = __ballot_sync(0xffffffffu, in); mask; mask &= mask - 1) {
+            const int j = __ffs(mask) - 1;
+            const int b = __shfl_sync(0xffffffffu, kb, j);
+            int t = __shfl_sync(0xffffffffu, xo, j) + lane;
+            if (t > 2 * R) t -= G.nx;
+            if ((unsigned)t <= (unsigned)(2 * R)) {
+                const float2* __restrict__ k2 = reinterpret_cast<const float2*>(K + b + 6 * t);
+                const float2 a = k2[0], bb = k2[1], c = k2[2];
+                const float k[6] = {a.x, a.y, bb.x, bb.y, c.x, c.y};
+                pull_add<PB>(acc, sd + (q0 + j) * sd_stride, k);
+            }
+        }
+    }
+}
+
+// One tile of the particles p0 .. p0 + fine_parts(PB, SUB) - 1 (those below
+// ne) from their SOAR fields so_g [ne][N_R].  PULL: smem is
+// fine_list_bytes(cap, ...) with cap >= the tile's list length, followed by the stencil's 6 (2R +
+// 1)^2 floats if k_smem: it is copied there when the tile's list is long
+// enough to reuse it (every observation of a row reads it at another offset,
+// and the state's stream through L1 evicts it).
+// Called by whole CTAs of NTHREADS threads; a CTA may call it for several
+// tiles in turn.
+template <bool PULL, int PB, int SUB>
+__device__ __forceinline__ void fine_cta(const QhalfArgs& A, const Grid& G, const Coarse& C, int tile, int p0,
+                                         const float* __restrict__ so_g, float* smem, int cap, bool k_smem)
+{
+    constexpr int PARTS = fine_parts(PB, SUB);
+    __shared__ FineRows rows;
+    const int ntx = (G.nx + FINE_TX - 1) / FINE_TX;
+    const int x0 = (tile % ntx) * FINE_TX, y0 = (tile / ntx) * FINE_TY;
+    const int np = min(PARTS, G.ne - p0), tid = threadIdx.x, lane = tid & 31;
+    int2* const off = reinterpret_cast<int2*>(smem + 2 * (size_t)cap * PARTS);
+    float* const sK = smem + 2 * (size_t)cap * (PARTS + 1);
+    __syncthreads();                         // a previous tile's readers are done
+    for (int i = tid; i < FINE_TY + 2; i += NTHREADS) {
+        float t, w[4];
+        rows.b[i] = coarse_interval(y0 - 1 + i, C.nRy, C.c, C.o, G.ny, t);
+        cubic_weights(t, w);
+        rows.w[i] = make_float4(w[0], w[1], w[2], w[3]);
+    }
+    int n = 0;
+    bool copied = false;
+    if (PULL) {
+        // the minimum-image offset of the tile origin from each listed
+        // observation, in (-n/2, n/2] (the cells add theirs, at most one
+        // period above), and the particles' S d
+        n = min(min(A.tile_cnt[tile], MAX_TILE_OBS), cap);
+        copied = k_smem && n >= 4;
+        if (copied)
+            for (int k = tid; k < 6 * (2 * A.R + 1) * (2 * A.R + 1); k += NTHREADS) sK[k] = A.K[k];
+        for (int q = tid; q < n; q += NTHREADS) {
+            const int l = A.tile_obs[tile * A.tile_cap + q];
+            int dx = pmod(x0 - A.obs_cell[2 * l], G.nx), dy = pmod(y0 - A.obs_cell[2 * l + 1], G.ny);
+            if (dx > G.nx / 2) dx -= G.nx;
+            if (dy > G.ny / 2) dy -= G.ny;
+            off[q] = make_int2(dx, dy);
+        }
+        for (int k = tid; k < n * PARTS; k += NTHREADS) {
+            const int q = k / PARTS, pp = k % PARTS;
+            const long long at = (long long)(p0 + min(pp, np - 1)) * 2 * A.nobs + 2 * A.tile_obs[tile * A.tile_cap + q];
+            float* const d = smem + 2 * q * PARTS + (PB == 1 ? 2 * pp : 4 * (pp >> 1) + (pp & 1));
+            d[0] = (float)A.Sd[at];
+            d[PB == 1 ? 1 : 2] = (float)A.Sd[at + 1];
         }
     }
     __syncthreads();
-    __shared__ int obs_ox[PULL ? MAX_TILE_OBS : 1], obs_oy[PULL ? MAX_TILE_OBS : 1];
-    __shared__ float obs_su[PULL ? MAX_TILE_OBS : 1], obs_sv[PULL ? MAX_TILE_OBS : 1];
-    const int n_obs_tile = PULL ? tile_obs_prep(A, G, x0, y0, p, tile, obs_ox, obs_oy, obs_su, obs_sv) : 0;
-    float* __restrict__ U = (A.par[p] ? A.b1 : A.b0) + (long long)p * 3 * G.plane;
-    const int W = 2 * A.R + 1;
-    float m = 0.0f;    // CFL rate max of the updated cells (with A.amax)
-    if (PULL && n_obs_tile > 0) {
-        // Pull by observation: each observation of the list, in list order,
-        // adds its stencil to the cells it reaches (up to two column and two
-        // row intervals of the tile, split where the minimum image wraps),
-        // with a barrier between observations.  Every cell thus receives the
-        // same operations in the same order as in the per-cell loop below,
-        // without testing the observations that do not reach it.  The
-        // stencil's reach 2R + 1 lies within the grid on both axes (iewpf_create
-        // refuses smaller grids), so each cell sees one image of each stencil.
-        static_assert(TX * TY % NTHREADS == 0, "whole tiles per thread");
-        constexpr int PER = TX * TY / NTHREADS, N = TX * TY;
-        float v0[PER], v1[PER], v2[PER];
+    const int warp = tid >> 5, grp = warp / STRIPS, sx = 32 * (warp % STRIPS);
+    constexpr int ROWS = FINE_TY / SUB;
+    const int r0 = (grp % SUB) * ROWS, r1 = r0 + ROWS, g0 = (grp / SUB) * PB;
+    if (x0 + sx >= G.nx || y0 + r0 >= G.ny || g0 >= np) return;      // uniform over the warp
+    const long long NR = (long long)C.nRx * C.nRy;
+    const int x = x0 + sx + lane;
+    const bool valid = x < G.nx;
+    int a, ha;
+    float wx[4], hw[4];
+    column_taps(x, G, C, a, wx);
+    column_taps((lane & 1) ? x0 + sx + 32 : x0 + sx - 1, G, C, ha, hw);
+    // the coarse columns a0 - 1 .. a0 + 30 by lane, if they hold the strip's taps
+    const int a0 = __shfl_sync(0xffffffffu, a, 0);
+    const bool by_lane = __shfl_sync(0xffffffffu, a, 31) + 2 <= a0 + 30;
+    const int mycol = pmod(a0 - 1 + lane, C.nRx);
+    int hc[4];
 #pragma unroll
-        for (int k = 0; k < PER; ++k) {
-            const int i = tid + k * NTHREADS;
-            const int fx = i % TX + 1, fy = i / TX + 1;
-            v0[k] = deta[fy][fx];
-            v1[k] = -G.sgh * (deta[fy + 1][fx] - deta[fy - 1][fx]) * G.inv_2dy;
-            v2[k] = G.sgh * (deta[fy][fx + 1] - deta[fy][fx - 1]) * G.inv_2dx;
+    for (int k = 0; k < 4; ++k) hc[k] = pmod(ha - 1 + k, C.nRx);
+    // coarse row of an extended index (at most a few rows beyond the grid)
+    auto wrap_row = [&](int bk) { return bk < 0 ? bk + C.nRy : (bk >= C.nRy ? bk - C.nRy : bk); };
+    const float* __restrict__ hso = so_g + (long long)(p0 + min(g0 + min(lane >> 1, PB - 1), np - 1)) * NR;
+    const int last = np - 1 - g0;            // particles beyond np repeat the last and are not stored
+    const float* so_p[PB];
+#pragma unroll
+    for (int pp = 0; pp < PB; ++pp) so_p[pp] = so_g + (long long)(p0 + g0 + min(pp, last)) * NR;
+    float R[4][PB], hR[4], raw[PB], hraw[4];
+    auto request = [&](int bk) {             // coarse row bk
+        const int o = wrap_row(bk) * C.nRx;      // within one particle's coarse grid
+        if (by_lane) {
+#pragma unroll
+            for (int pp = 0; pp < PB; ++pp) raw[pp] = so_p[pp][o + mycol];
         }
-        __syncthreads();
-        float* __restrict__ acc = pool;     // [3][TY][TX]
 #pragma unroll
-        for (int k = 0; k < PER; ++k) {
-            const int i = tid + k * NTHREADS;
-            acc[i] = v0[k];
-            acc[N + i] = v1[k];
-            acc[2 * N + i] = v2[k];
+        for (int k = 0; k < 4; ++k) hraw[k] = hso[o + hc[k]];
+    };
+    auto take = [&](int k, int bk) {         // into R[k]
+        if (by_lane) {
+#pragma unroll
+            for (int pp = 0; pp < PB; ++pp)
+                R[k][pp] = taps(wx, __shfl_sync(0xffffffffu, raw[pp], a - a0), __shfl_sync(0xffffffffu, raw[pp], a - a0 + 1),
+                                __shfl_sync(0xffffffffu, raw[pp], a - a0 + 2), __shfl_sync(0xffffffffu, raw[pp], a - a0 + 3));
+        } else {
+            const int o = wrap_row(bk) * C.nRx;
+            const int c0 = pmod(a - 1, C.nRx), c1 = pmod(a, C.nRx), c2 = pmod(a + 1, C.nRx), c3 = pmod(a + 2, C.nRx);
+#pragma unroll
+            for (int pp = 0; pp < PB; ++pp) {
+                const float* __restrict__ q = so_p[pp] + o;
+                R[k][pp] = taps(wx, q[c0], q[c1], q[c2], q[c3]);
+            }
         }
-        __syncthreads();
-        const int txv = min(TX, G.nx - x0), tyv = min(TY, G.ny - y0);
-        const int fs = W * W;
-        for (int q = 0; q < n_obs_tile; ++q) {
-            const int ox0 = obs_ox[q], oy0 = obs_oy[q];
-            const float su = obs_su[q], sv = obs_sv[q];
-            // cells tx with the offset ox0 + tx in [-R, R], or ox0 + tx - n
-            // in [-R, R] past the wrap (offset at the interval's start)
-            const int xa[2] = {max(0, -A.R - ox0), max(0, G.nx - A.R - ox0)};
-            const int xb[2] = {min(txv, A.R - ox0 + 1), min(txv, G.nx + A.R - ox0 + 1)};
-            const int ya[2] = {max(0, -A.R - oy0), max(0, G.ny - A.R - oy0)};
-            const int yb[2] = {min(tyv, A.R - oy0 + 1), min(tyv, G.ny + A.R - oy0 + 1)};
+        hR[k] = taps(hw, hraw[0], hraw[1], hraw[2], hraw[3]);
+    };
+    int b = rows.b[r0];
 #pragma unroll
-            for (int ix = 0; ix < 2; ++ix) {
-                const int w = xb[ix] - xa[ix];
-                if (w <= 0) continue;
-                const int oxa = ox0 + xa[ix] - (ix ? G.nx : 0) + A.R;
+    for (int k = 0; k < 4; ++k) {
+        request(b - 1 + k);
+        take(k, b - 1 + k);
+    }
+    request(b + 3);
+    // the state at column x of the row to write
+    float* U[PB];
 #pragma unroll
-                for (int iy = 0; iy < 2; ++iy) {
-                    const int h = yb[iy] - ya[iy];
-                    if (h <= 0) continue;
-                    const int oya = oy0 + ya[iy] - (iy ? G.ny : 0) + A.R;
-                    // the rectangle's w x h cells, linearised over the CTA;
-                    // row = floor((i + 1/2) / w) in float is exact here
-                    // (w, h <= 2R + 1, far below float's integer range)
-                    const float rw = 1.0f / (float)w;
-                    for (int i = tid; i < w * h; i += NTHREADS) {
-                        const int ry = __float2int_rz(((float)i + 0.5f) * rw);
-                        const int rx = i - ry * w;
-                        const int o = (oya + ry) * W + oxa + rx;
-                        const int c = (ya[iy] + ry) * TX + xa[ix] + rx;
-                        acc[c] = fmaf(sv, A.K[3 * fs + o], fmaf(su, A.K[0 * fs + o], acc[c]));
-                        acc[N + c] = fmaf(sv, A.K[4 * fs + o], fmaf(su, A.K[1 * fs + o], acc[N + c]));
-                        acc[2 * N + c] = fmaf(sv, A.K[5 * fs + o], fmaf(su, A.K[2 * fs + o], acc[2 * N + c]));
+    for (int pp = 0; pp < PB; ++pp) {
+        const int p = p0 + g0 + min(pp, last);
+        U[pp] = (A.par[p] ? A.b1 : A.b0) + (long long)p * 3 * G.plane + (long long)(y0 + r0) * G.nx + (valid ? x : 0);
+    }
+    float dm[PB], d0[PB], dn[PB], hd = 0.0f, m[PB];
+#pragma unroll
+    for (int pp = 0; pp < PB; ++pp) dm[pp] = d0[pp] = m[pp] = 0.0f;
+    for (int i = r0; i < r1 + 2; ++i) {
+        const int ty = i - 2, gy = y0 + ty;          // the row to write
+        if (gy >= G.ny) break;
+        const bool write = ty >= r0;
+        float u[3][PB];                              // (requested first, used last)
+        if (write) {
+#pragma unroll
+            for (int pp = 0; pp < PB; ++pp)
+#pragma unroll
+                for (int f = 0; f < 3; ++f) u[f][pp] = U[pp][f * G.plane];
+        }
+        // field of row y0 + i - 1
+        if (rows.b[i] != b) {
+            b = rows.b[i];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+#pragma unroll
+                for (int pp = 0; pp < PB; ++pp) R[k][pp] = R[k + 1][pp];
+                hR[k] = hR[k + 1];
+            }
+            take(3, b + 2);
+            request(b + 3);
+        }
+        const float4 w4 = rows.w[i];
+        const float w[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+        for (int pp = 0; pp < PB; ++pp) dn[pp] = taps(w, R[0][pp], R[1][pp], R[2][pp], R[3][pp]);
+        const float hn = taps(w, hR[0], hR[1], hR[2], hR[3]);
+        if (write) {
+            float acc[3][PB];
+#pragma unroll
+            for (int pp = 0; pp < PB; ++pp) {
+                const float hl = __shfl_sync(0xffffffffu, hd, 2 * pp), hr = __shfl_sync(0xffffffffu, hd, 2 * pp + 1);
+                float l = __shfl_up_sync(0xffffffffu, d0[pp], 1), r = __shfl_down_sync(0xffffffffu, d0[pp], 1);
+                if (lane == 0) l = hl;
+                if (lane == 31) r = hr;
+                acc[0][pp] = d0[pp];
+                acc[1][pp] = -G.sgh * (dn[pp] - dm[pp]) * G.inv_2dy;
+                acc[2][pp] = G.sgh * (r - l) * G.inv_2dx;
+            }
+            if (PULL) {
+                if (copied) pull_row<PB>(acc, G, A.R, off, n, smem + 2 * g0, 2 * PARTS, sK, ty, sx);
+                else pull_row<PB>(acc, G, A.R, off, n, smem + 2 * g0, 2 * PARTS, A.K, ty, sx);
+            }
+            if (valid) {
+#pragma unroll
+                for (int pp = 0; pp < PB; ++pp) {
+                    if (pp <= last) {
+                        const float e1 = u[0][pp] + acc[0][pp], u1 = u[1][pp] + acc[1][pp], v1 = u[2][pp] + acc[2][pp];
+                        U[pp][0] = e1;
+                        U[pp][G.plane] = u1;
+                        U[pp][2 * G.plane] = v1;
+                        if (A.amax) m[pp] = fmaxf(m[pp], cfl_of(e1, u1, v1, G));
                     }
                 }
             }
-            __syncthreads();
+#pragma unroll
+            for (int pp = 0; pp < PB; ++pp) U[pp] += G.nx;
         }
 #pragma unroll
-        for (int k = 0; k < PER; ++k) {
-            const int i = tid + k * NTHREADS;
-            const int gx = x0 + i % TX, gy = y0 + i / TX;
-            if (gx >= G.nx || gy >= G.ny) continue;
-            const long long g = (long long)gy * G.nx + gx;
-            const float e1 = U[g] + acc[i], u1 = U[G.plane + g] + acc[N + i], v1 = U[2 * G.plane + g] + acc[2 * N + i];
-            U[g] = e1;
-            U[G.plane + g] = u1;
-            U[2 * G.plane + g] = v1;
-            if (A.amax) m = fmaxf(m, cfl_of(e1, u1, v1, G));
+        for (int pp = 0; pp < PB; ++pp) {
+            dm[pp] = d0[pp];
+            d0[pp] = dn[pp];
         }
-    } else
-    for (int i = tid; i < TX * TY; i += NTHREADS) {
-        const int tx = i % TX, ty = i / TX;
-        const int gx = x0 + tx, gy = y0 + ty;
-        if (gx >= G.nx || gy >= G.ny) continue;
-        const int fx = tx + 1, fy = ty + 1;
-        float de = deta[fy][fx];
-        float dhu = -G.sgh * (deta[fy + 1][fx] - deta[fy - 1][fx]) * G.inv_2dy;
-        float dhv = G.sgh * (deta[fy][fx + 1] - deta[fy][fx - 1]) * G.inv_2dx;
-        const long long g = (long long)gy * G.nx + gx;
-        const float e1 = U[g] + de, u1 = U[G.plane + g] + dhu, v1 = U[2 * G.plane + g] + dhv;
-        U[g] = e1;
-        U[G.plane + g] = u1;
-        U[2 * G.plane + g] = v1;
-        if (A.amax) m = fmaxf(m, cfl_of(e1, u1, v1, G));
+        hd = hn;
     }
     if (A.amax) {
-        __shared__ float red[NTHREADS / 32];
-        m = warp_max(m);
-        if ((tid & 31) == 0) red[tid >> 5] = m;
-        __syncthreads();
-        if (tid < 32) {
-            float v = tid < NTHREADS / 32 ? red[tid] : 0.0f;
-            v = warp_max(v);
+#pragma unroll
+        for (int pp = 0; pp < PB; ++pp) {
+            const float v = warp_max(m[pp]);
             // non-negative floats order like their bit patterns
-            if (tid == 0) atomicMax(reinterpret_cast<int*>(A.amax) + p, __float_as_int(v));
+            if (lane == 0 && pp <= last) atomicMax(reinterpret_cast<int*>(A.amax) + p0 + g0 + pp, __float_as_int(v));
         }
     }
 }

@@ -57,6 +57,37 @@ def test_random_vectors_over_philox_blocks(nx, ny):
     assert rel_l2(ens.get_state(), ref) <= 1e-5
 
 
+
+# particles per CTA of the fine stage: 1, 4 and 16 (the largest groups the ensemble fills the GPU with)
+@pytest.mark.parametrize("ne", [3, 305, 1233])
+@pytest.mark.parametrize("nx,ny,c", [(48, 50, 3), (65, 47, 1), (97, 75, 5)])
+def test_fine_stage_groups_and_tile_edges(nx, ny, c, ne):
+    """Analysis update and Q^{1/2} on grids that do not fill their 64 x 32 tiles and 32-column strips, with
+    observations whose stencils wrap both seams, for every particle grouping; sampled particles (first,
+    last, group edges) against the oracle at 1e-5."""
+    cfg = synth.Config("edge", nx, ny, n_particles=ne, n_obs=3, c_omega=c)
+    ens, P = ensemble(cfg), oracle_problem(cfg)
+    base = synth.initial_state(cfg, 7, seed=7).astype(np.float32)
+    U32 = base[np.arange(ne) % 7]
+    ens.set_state(U32)
+    xy = np.array([[0.2 * cfg.dx, 0.4 * cfg.dy], [(nx - 0.5) * cfg.dx, 0.5 * ny * cfg.dy], [33.5 * cfg.dx, 32.5 * cfg.dy]])
+    cells = [O.obs_cell(P, *p) for p in xy]
+    y = synth.obs_from_state(cfg, synth.initial_state(cfg, 1, seed=3)[0], np.array(cells), synth.obs_noise(cfg, 3, 0))
+    d = ens.assimilate(xy, y)
+    got = ens.get_state()
+    sample = sorted({0, ne - 1, min(ne - 1, 3), min(ne - 1, 4), min(ne - 1, 15), min(ne - 1, 16), ne // 2})
+    for i in sample:
+        ref, _ = O.assimilate(P, U32[i:i + 1].astype(np.float64), cells, y, t=0, p0=i,
+                              scalars={"beta": d["beta"], "alpha": d["alpha"][i:i + 1]})
+        assert rel_l2(got[i], ref[0]) <= 1e-5
+    x = np.random.default_rng(3).standard_normal((ne, P.N_R)).astype(np.float32)
+    ens.set_state(U32)
+    ens.add_qhalf(x)
+    got = ens.get_state()
+    for i in sample:
+        assert rel_l2(got[i], O.add_qhalf(P, x[i].astype(np.float64), U32[i].astype(np.float64))) <= 1e-5
+
+
 @pytest.mark.parametrize("nx,ny", [(44, 46), (64, 64), (66, 47), (96, 45), (93, 50), (97, 44), (176, 48)])
 def test_marching_shapes_agree_bitwise_and_with_the_oracle(nx, ny):
     """Rows that close on a ring of lanes (44, 64, 96, 93 with 3 columns, 66) or take strips with halo (one
