@@ -414,8 +414,11 @@ IEWPF_API int iewpf_set_stepper(iewpf_ctx_t* ctx, int kind, int nc, int rows, in
 /* Autotuner: times every marching shape on the context's own problem (the
  * state is left unchanged) and keeps the fastest; shape[4] (may be NULL)
  * receives (kind, nc, rows, warps).  Runs by itself before the first
- * forecast unless iewpf_set_stepper was called.  get_stepper reads the
- * current shape.  Errors: EINVAL, ECUDA. */
+ * forecast unless iewpf_set_stepper was called.  It also times whole model
+ * steps with each particle resident in the shared memory of a thread-block
+ * cluster, where the grid is small enough; forecasts without drifters then
+ * use them if faster (same bits; iewpf_set_stepper turns them off).
+ * get_stepper reads the current shape.  Errors: EINVAL, ECUDA. */
 IEWPF_API int iewpf_tune(iewpf_ctx_t* ctx, int* shape);
 IEWPF_API int iewpf_get_stepper(const iewpf_ctx_t* ctx, int* shape);
 

@@ -148,12 +148,15 @@ struct iewpf_ctx {
     unsigned int* h_iters = nullptr;
     cudaStream_t st2 = nullptr;
     struct FcGraph {
-        int n, err, fixed, have, nd, stepper, nc, TH, warps, paired;
+        int n, err, fixed, have, nd, stepper, nc, TH, warps, paired, resident;
         cudaGraphExec_t exec;
         int64_t launches_fixed, launches_per_iter;
     };
     std::vector<FcGraph> fgraphs;
     MarchShape shape{2, 64, 4};
+    // CTAs per particle of the resident model step (resident.cu) that the tuner
+    // found faster than the marched scheme steps; 0: none
+    int resident = 0;
     bool tuned = false;
     std::string err;
 };
@@ -439,6 +442,29 @@ int tune_stepper(iewpf_ctx* ctx)
     const MarchShape at4 = best_shape;
     for (int w : {2, 8})
         if (!rc) rc = probe(MarchShape{at4.nc, at4.TH, w, at4.paired});
+    // the resident model step, 16 scheme steps a probe, against 16 of the best
+    // march with the loop control of a captured forecast (5 us a scheme step)
+    ctx->resident = 0;
+    float per_step = best / 3.0f + 0.005f;
+    auto probe_resident = [&](int cl) -> int {
+        for (int r = 0; r < 2; ++r) {
+            if (r) CK(cudaEventRecord(a, ctx->st));
+            CK(launch_resident(ctx->buf[0], ctx->buf[1], ctx->par, ctx->amax, ctx->nsub, ctx->dtp, ctx->G, ctx->P.courant,
+                               ctx->P.dt_model, 16, ctx->work, ctx->flag, cl, 0, ctx->st));
+        }
+        CK(cudaEventRecord(b, ctx->st));
+        CK(cudaEventSynchronize(b));
+        float ms = 0.0f;
+        CK(cudaEventElapsedTime(&ms, a, b));
+        ctx->launches += 2;
+        if (ms / 16.0f < per_step) {
+            per_step = ms / 16.0f;
+            ctx->resident = cl;
+        }
+        return IEWPF_OK;
+    };
+    for (int cl : {2, 4, 8})
+        if (!rc && resident_fits(ctx->G.nx, ctx->G.ny, cl)) rc = probe_resident(cl);
     cudaEventDestroy(a);
     cudaEventDestroy(b);
     if (rc) return rc;
@@ -494,9 +520,11 @@ int read_flags(iewpf_ctx* ctx)
 // Captures n_steps model steps into one executable graph: per model step the
 // CFL pass, a conditional WHILE node whose body is one scheme step (with the
 // drifters) and the loop control reading the largest n_sub on the device, the
-// parity flip, and the model error.  The scheme-step index and the model-step
-// counter come from device memory, so the graph serves every call with the
-// same pattern and needs no host synchronisation between model steps.
+// parity flip, and the model error; or, without drifters where the tuner found
+// it faster, the CFL pass, the resident model step and the model error.  The
+// scheme-step index and the first model step's counter come from device
+// memory, so the graph serves every call with the same pattern and needs no
+// host synchronisation between model steps.
 static cudaError_t capture_forecast(iewpf_ctx* ctx, int n_steps, int add_err, int fixed, bool have0,
                                     iewpf_ctx::FcGraph& fg)
 {
@@ -505,49 +533,63 @@ static cudaError_t capture_forecast(iewpf_ctx* ctx, int n_steps, int add_err, in
     if (e != cudaSuccess) return e;
     int64_t fixed_launches = 0;
     const int64_t per_iter = 2 + (ctx->nd > 0 ? 1 : 0);
+    const int resident = fg.resident;
     bool have = have0;
     auto body = [&]() -> cudaError_t {
         cudaError_t r;
         for (int k = 0; k < n_steps; ++k) {
-            if ((r = launch_cfl(ctx->buf[0], ctx->buf[1], ctx->par, ctx->amax, ctx->nsub, ctx->dtp, ctx->maxsub,
-                                ctx->G, ctx->P.courant, ctx->P.dt_model, fixed, st, have, ctx->flag)) != cudaSuccess)
-                return r;
-            fixed_launches += (fixed > 0 || have) ? 1 : 2;
-            if ((r = launch_step_reset(ctx->d_s, st)) != cudaSuccess) return r;
-            fixed_launches += 1;
-            cudaStreamCaptureStatus status;
-            cudaGraph_t g = nullptr;
-            const cudaGraphNode_t* deps = nullptr;
-            size_t ndeps = 0;
-            if ((r = cudaStreamGetCaptureInfo(st, &status, nullptr, &g, &deps, nullptr, &ndeps)) != cudaSuccess)
-                return r;
-            cudaGraphConditionalHandle h;
-            if ((r = cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault)) != cudaSuccess) return r;
-            cudaGraphNodeParams prm = {};
-            prm.type = cudaGraphNodeTypeConditional;
-            prm.conditional.handle = h;
-            prm.conditional.type = cudaGraphCondTypeWhile;
-            prm.conditional.size = 1;
-            cudaGraphNode_t node;
-            if ((r = cudaGraphAddNode(&node, g, deps, nullptr, ndeps, &prm)) != cudaSuccess) return r;
-            cudaGraph_t loop = prm.conditional.phGraph_out[0];
-            if ((r = cudaStreamUpdateCaptureDependencies(st, &node, nullptr, 1, cudaStreamSetCaptureDependencies)) !=
-                cudaSuccess)
-                return r;
-            if ((r = cudaStreamBeginCaptureToGraph(st2, loop, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal)) !=
-                cudaSuccess)
-                return r;
-            cudaError_t rb = launch_rk2_march(ctx->buf[0], ctx->buf[1], ctx->par, ctx->nsub, ctx->dtp, 0, ctx->G,
-                                              ctx->shape, st2, ctx->d_s);
-            if (rb == cudaSuccess && ctx->nd > 0)
-                rb = launch_drift(ctx->buf[0], ctx->buf[1], ctx->par, ctx->nsub, ctx->dtp, ctx->d_xy, ctx->nd, 0,
-                                  ctx->G, ctx->P.dx, ctx->P.dy, st2, ctx->d_s);
-            if (rb == cudaSuccess) rb = launch_step_ctl(ctx->d_s, ctx->maxsub, h, ctx->d_iters, st2);
-            r = cudaStreamEndCapture(st2, &loop);
-            if (rb != cudaSuccess) return rb;
-            if (r != cudaSuccess) return r;
-            if ((r = launch_par_update(ctx->par, ctx->nsub, ctx->G.ne, ctx->work, st)) != cudaSuccess) return r;
-            fixed_launches += 1;
+            if (resident) {
+                if (fixed <= 0 && !have) {
+                    if ((r = launch_cfl_rates(ctx->buf[0], ctx->buf[1], ctx->par, ctx->amax, ctx->G, st)) != cudaSuccess)
+                        return r;
+                    fixed_launches += 1;
+                }
+                if ((r = launch_resident(ctx->buf[0], ctx->buf[1], ctx->par, ctx->amax, ctx->nsub, ctx->dtp, ctx->G,
+                                         ctx->P.courant, ctx->P.dt_model, fixed, ctx->work, ctx->flag, resident, 1, st)) !=
+                    cudaSuccess)
+                    return r;
+                fixed_launches += 1;
+            } else {
+                if ((r = launch_cfl(ctx->buf[0], ctx->buf[1], ctx->par, ctx->amax, ctx->nsub, ctx->dtp, ctx->maxsub,
+                                    ctx->G, ctx->P.courant, ctx->P.dt_model, fixed, st, have, ctx->flag)) != cudaSuccess)
+                    return r;
+                fixed_launches += (fixed > 0 || have) ? 1 : 2;
+                if ((r = launch_step_reset(ctx->d_s, st)) != cudaSuccess) return r;
+                fixed_launches += 1;
+                cudaStreamCaptureStatus status;
+                cudaGraph_t g = nullptr;
+                const cudaGraphNode_t* deps = nullptr;
+                size_t ndeps = 0;
+                if ((r = cudaStreamGetCaptureInfo(st, &status, nullptr, &g, &deps, nullptr, &ndeps)) != cudaSuccess)
+                    return r;
+                cudaGraphConditionalHandle h;
+                if ((r = cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault)) != cudaSuccess) return r;
+                cudaGraphNodeParams prm = {};
+                prm.type = cudaGraphNodeTypeConditional;
+                prm.conditional.handle = h;
+                prm.conditional.type = cudaGraphCondTypeWhile;
+                prm.conditional.size = 1;
+                cudaGraphNode_t node;
+                if ((r = cudaGraphAddNode(&node, g, deps, nullptr, ndeps, &prm)) != cudaSuccess) return r;
+                cudaGraph_t loop = prm.conditional.phGraph_out[0];
+                if ((r = cudaStreamUpdateCaptureDependencies(st, &node, nullptr, 1, cudaStreamSetCaptureDependencies)) !=
+                    cudaSuccess)
+                    return r;
+                if ((r = cudaStreamBeginCaptureToGraph(st2, loop, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal)) !=
+                    cudaSuccess)
+                    return r;
+                cudaError_t rb = launch_rk2_march(ctx->buf[0], ctx->buf[1], ctx->par, ctx->nsub, ctx->dtp, 0, ctx->G,
+                                                  ctx->shape, st2, ctx->d_s);
+                if (rb == cudaSuccess && ctx->nd > 0)
+                    rb = launch_drift(ctx->buf[0], ctx->buf[1], ctx->par, ctx->nsub, ctx->dtp, ctx->d_xy, ctx->nd, 0,
+                                      ctx->G, ctx->P.dx, ctx->P.dy, st2, ctx->d_s);
+                if (rb == cudaSuccess) rb = launch_step_ctl(ctx->d_s, ctx->maxsub, h, ctx->d_iters, st2);
+                r = cudaStreamEndCapture(st2, &loop);
+                if (rb != cudaSuccess) return rb;
+                if (r != cudaSuccess) return r;
+                if ((r = launch_par_update(ctx->par, ctx->nsub, ctx->G.ne, ctx->work, st)) != cudaSuccess) return r;
+                fixed_launches += 1;
+            }
             if (add_err) {
                 QhalfArgs A{};
                 A.b0 = ctx->buf[0];
@@ -556,19 +598,19 @@ static cudaError_t capture_forecast(iewpf_ctx* ctx, int n_steps, int add_err, in
                 A.wtab = ctx->d_wtab;
                 A.from_philox = 1;
                 A.seed = ctx->P.seed;
-                A.t = 0;
+                A.t = (uint32_t)k;
                 A.t_dev = ctx->d_step;
                 A.stream = 0u + 16u * (uint32_t)ctx->P.instance_id;
                 A.xi_buf = ctx->d_xi;
                 A.soar_buf = ctx->d_soar;
                 A.amax = ctx->amax;
-                if ((r = cudaMemsetAsync(ctx->amax, 0, sizeof(float) * ctx->G.ne, st)) != cudaSuccess) return r;
+                // (the resident step leaves the rates cleared)
+                if (!resident && (r = cudaMemsetAsync(ctx->amax, 0, sizeof(float) * ctx->G.ne, st)) != cudaSuccess)
+                    return r;
                 if ((r = launch_qhalf(A, ctx->G, ctx->C, st)) != cudaSuccess) return r;
                 fixed_launches += qhalf_launches(A);
             }
             have = add_err && fixed <= 0;
-            if ((r = launch_counter_inc(ctx->d_step, st)) != cudaSuccess) return r;
-            fixed_launches += 1;
         }
         return cudaSuccess;
     };
@@ -593,12 +635,13 @@ int forecast_impl(iewpf_ctx* ctx, int n_steps, int add_err, int fixed)
     if (n_steps > 0) {
         const int have = ctx->cfl_ready && fixed <= 0;
         iewpf_ctx::FcGraph key{n_steps, add_err ? 1 : 0, fixed, have, ctx->nd, ctx->stepper, ctx->shape.nc,
-                               ctx->shape.TH, ctx->shape.warps, ctx->shape.paired, nullptr, 0, 0};
+                               ctx->shape.TH, ctx->shape.warps, ctx->shape.paired, ctx->nd > 0 ? 0 : ctx->resident,
+                               nullptr, 0, 0};
         iewpf_ctx::FcGraph* fg = nullptr;
         for (auto& g : ctx->fgraphs)
             if (g.n == key.n && g.err == key.err && g.fixed == key.fixed && g.have == key.have && g.nd == key.nd &&
                 g.stepper == key.stepper && g.nc == key.nc && g.TH == key.TH && g.warps == key.warps &&
-                g.paired == key.paired)
+                g.paired == key.paired && g.resident == key.resident)
                 fg = &g;
         if (!fg) {
             if (ctx->fgraphs.size() >= 8) {
@@ -1618,6 +1661,7 @@ int iewpf_set_stepper(iewpf_ctx_t* ctx, int kind, int nc, int rows, int warps)
         return fail(ctx, IEWPF_EINVAL, "bad stepper shape");
     ctx->stepper = kind;
     ctx->shape = MarchShape{nc, rows, warps, kind == 2};
+    ctx->resident = 0;
     ctx->tuned = true;
     return IEWPF_OK;
 }

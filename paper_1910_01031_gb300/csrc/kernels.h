@@ -11,6 +11,9 @@
 namespace iewpf {
 
 // ---- stepper.cu -----------------------------------------------------------
+// the CFL rates of the current state into amax
+cudaError_t launch_cfl_rates(const float* b0, const float* b1, const int* par, float* amax, const Grid& G,
+                             cudaStream_t st);
 // have_amax: amax already holds the CFL rates of the current state (left by
 // the model-error or analysis update); only n_sub is derived then
 cudaError_t launch_cfl(const float* b0, const float* b1, const int* par, float* amax, int* nsub, float* dtp,
@@ -20,14 +23,13 @@ cudaError_t launch_cfl(const float* b0, const float* b1, const int* par, float* 
 cudaError_t launch_par_update(int* par, const int* nsub, int ne, unsigned long long* work, cudaStream_t st);
 // the scheme-step loop of a captured model step: reset the index, then after
 // every step advance it and keep looping while it is below the largest n_sub
-// (and below kMaxSubSingle); the model-step counter of the model error
+// (and below kMaxSubSingle)
 constexpr int kMaxSubSingle = 100000;
 // fixed observation layouts from this size on are factored in a nested-dissection order
 constexpr int kNdMinObs = 256;
 cudaError_t launch_step_reset(int* s_dev, cudaStream_t st);
 cudaError_t launch_step_ctl(int* s_dev, const int* maxsub, cudaGraphConditionalHandle h, unsigned int* iters,
                             cudaStream_t st);
-cudaError_t launch_counter_inc(uint32_t* t_dev, cudaStream_t st);
 // s_dev (may be null): the scheme-step index read from device memory instead of s
 cudaError_t launch_drift(const float* b0, const float* b1, const int* par, const int* nsub, const float* dtp,
                          double* xy, int nd, int s, const Grid& G, double dx, double dy, cudaStream_t st,
@@ -99,6 +101,16 @@ cudaError_t launch_rk2_march(float* b0, float* b1, const int* par, const int* ns
                              const Grid& G, const MarchShape& shape, cudaStream_t st,
                              const int* s_dev = nullptr);
 
+// ---- resident.cu ----------------------------------------------------------
+// one model step of every particle in one launch, a cluster of cl CTAs per
+// particle (resident_fits: whether the grid's slabs fit); n_sub from amax (or
+// fixed) as nsub_kernel, the state rewritten in place, amax cleared, the work
+// counted.  store = 0 changes nothing (timing).
+bool resident_fits(int nx, int ny, int cl);
+cudaError_t launch_resident(float* b0, float* b1, const int* par, float* amax, int* nsub, float* dtp, const Grid& G,
+                            double courant, double dt_model, int fixed, unsigned long long* work, int* flag, int cl,
+                            int store, cudaStream_t st);
+
 // ---- qhalf.cu -------------------------------------------------------------
 // psi += Q^{1/2} x (+ the optimal-proposal pull) for every particle.
 struct QhalfArgs {
@@ -110,7 +122,7 @@ struct QhalfArgs {
     int from_philox;
     uint64_t seed;
     uint32_t t;
-    const uint32_t* t_dev;    // if set, the draw counter is read from device memory
+    const uint32_t* t_dev;    // if set, the draw counter is t beyond the one in device memory
     uint32_t stream;
     const float* x;           // [ne][N_R]
     // optimal-proposal pull (may be disabled)

@@ -16,7 +16,7 @@ __global__ void coarse_normals_kernel(QhalfArgs A, long long NR)
     const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (4 * q >= NR) return;
     const int p = blockIdx.y;
-    const uint32_t t = A.t_dev ? *A.t_dev : A.t;
+    const uint32_t t = (A.t_dev ? *A.t_dev : 0u) + A.t;
     qhalf::normals_block(seed_key(A.seed), (uint32_t)p, t, A.stream, (uint32_t)q, NR, A.xi_buf + (long long)p * NR);
 }
 

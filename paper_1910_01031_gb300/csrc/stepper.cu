@@ -163,16 +163,24 @@ cudaError_t launch_drift_errors(const double* xy, const double* truth, int ne, i
     return cudaGetLastError();
 }
 
+cudaError_t launch_cfl_rates(const float* b0, const float* b1, const int* par, float* amax, const Grid& G,
+                             cudaStream_t st)
+{
+    cudaMemsetAsync(amax, 0, sizeof(float) * G.ne, st);
+    const long long blocks = (G.plane + NTHREADS * 8 - 1) / (NTHREADS * 8);
+    dim3 grid((unsigned)(blocks < 1 ? 1 : (blocks > 4096 ? 4096 : blocks)), G.ne);
+    cfl_kernel<<<grid, NTHREADS, 0, st>>>(b0, b1, par, amax, G);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_cfl(const float* b0, const float* b1, const int* par, float* amax, int* nsub, float* dtp,
                        int* maxsub, const Grid& G, double courant, double dt_model, int fixed,
                        cudaStream_t st, bool have_amax, int* flag)
 {
-    if (!have_amax) cudaMemsetAsync(amax, 0, sizeof(float) * G.ne, st);
     cudaMemsetAsync(maxsub, 0, sizeof(int), st);
     if (fixed <= 0 && !have_amax) {
-        const long long blocks = (G.plane + NTHREADS * 8 - 1) / (NTHREADS * 8);
-        dim3 grid((unsigned)(blocks < 1 ? 1 : (blocks > 4096 ? 4096 : blocks)), G.ne);
-        cfl_kernel<<<grid, NTHREADS, 0, st>>>(b0, b1, par, amax, G);
+        const cudaError_t e = launch_cfl_rates(b0, b1, par, amax, G, st);
+        if (e != cudaSuccess) return e;
     }
     nsub_kernel<<<(G.ne + 127) / 128, 128, 0, st>>>(amax, nsub, dtp, maxsub, G.ne, courant, dt_model, fixed, flag);
     return cudaGetLastError();
@@ -205,8 +213,6 @@ __global__ void step_ctl_kernel(int* s_dev, const int* maxsub, cudaGraphConditio
     if (iters) *iters += 1u;
     cudaGraphSetConditional(h, (s < *maxsub && s < kMaxSubSingle) ? 1u : 0u);
 }
-
-__global__ void counter_inc_kernel(uint32_t* t) { *t += 1u; }
 }  // namespace
 
 cudaError_t launch_step_reset(int* s_dev, cudaStream_t st)
@@ -219,12 +225,6 @@ cudaError_t launch_step_ctl(int* s_dev, const int* maxsub, cudaGraphConditionalH
                             cudaStream_t st)
 {
     step_ctl_kernel<<<1, 1, 0, st>>>(s_dev, maxsub, h, iters);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_counter_inc(uint32_t* t_dev, cudaStream_t st)
-{
-    counter_inc_kernel<<<1, 1, 0, st>>>(t_dev);
     return cudaGetLastError();
 }
 

@@ -110,3 +110,26 @@ def test_marching_shapes_agree_bitwise_and_with_the_oracle(nx, ny):
                     ref, _, _ = O.forecast(P, U64, 1, False, t0=0)
                     assert rel_l2(got, ref) <= 1e-5
                 assert np.array_equal(got, first), (kind, nc, rows, warps)
+
+
+@pytest.mark.parametrize("nx,ny,c", [(16, 17, 1), (33, 35, 1), (64, 64, 3), (50, 49, 3), (96, 45, 3), (128, 64, 3)])
+def test_resident_model_steps_equal_the_march(nx, ny, c):
+    """Grids small enough to stay in a cluster's shared memory (uneven slabs, rows of one to four blocks of
+    32 columns, more rows than warps): tuned forecasts, with and without model error and with a fixed number
+    of scheme steps, against the marched ones bit for bit, with the same counters of work and scheme steps."""
+    cfg = synth.Config("edge", nx, ny, n_particles=3, c_omega=c)
+    U32, _ = start_state(cfg, 3)
+    a, b = ensemble(cfg), ensemble(cfg)
+    shape = a.tune()
+    b.set_stepper(*shape)
+    for e in (a, b):
+        e.set_state(U32)
+    w0 = a.work()
+    for e in (a, b):
+        e.forecast(2, True)
+        e.forecast(1, False)
+        e.forecast_fixed(1, True, 14)
+    assert np.array_equal(a.get_state(), b.get_state())
+    assert np.array_equal(a.last_nsub(), b.last_nsub())
+    assert a.work() - w0 == b.work()
+    assert a.counters() == b.counters()
