@@ -273,28 +273,24 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmap_in, const __nv_bfloat16*
             } else {
                 uint32_t v[32];
                 tmem_ld32(ta, v);
-                __align__(16) __nv_bfloat162 hv[16];
+                uint4 out[4];
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const float z0 = __uint_as_float(v[2 * j]) + sbias[32 * h + 2 * j];
-                    const float z1 = __uint_as_float(v[2 * j + 1]) + sbias[32 * h + 2 * j + 1];
-                    hv[j] = __floats2bfloat162_rn(silu_act(z0), silu_act(z1));
+                for (int u = 0; u < 4; ++u) {
+                    __nv_bfloat162 hv[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int c = 8 * u + 2 * j;
+                        const float2 bb = *reinterpret_cast<const float2*>(sbias + 32 * h + c);
+                        hv[j] = __floats2bfloat162_rn(silu_act(__uint_as_float(v[c]) + bb.x),
+                                                      silu_act(__uint_as_float(v[c + 1]) + bb.y));
+                    }
+                    out[u] = make_uint4(*reinterpret_cast<uint32_t*>(&hv[0]), *reinterpret_cast<uint32_t*>(&hv[1]),
+                                        *reinterpret_cast<uint32_t*>(&hv[2]), *reinterpret_cast<uint32_t*>(&hv[3]));
                 }
-                // this pixel and its periodic images in the padded output
-                const size_t pw = (size_t)(nx + 2), plane = (size_t)(ny + 2) * pw;
-                const int ys[2] = {y + 1, y == 0 ? ny + 1 : (y == ny - 1 ? 0 : -1)};
-                const int xs[2] = {x + 1, x == 0 ? nx + 1 : (x == nx - 1 ? 0 : -1)};
-                const uint4* src = reinterpret_cast<const uint4*>(hv);
-#pragma unroll
-                for (int a = 0; a < 2; ++a)
-#pragma unroll
-                    for (int c = 0; c < 2; ++c)
-                        if (ys[a] >= 0 && xs[c] >= 0) {
-                            uint4* p = reinterpret_cast<uint4*>(
-                                aout + ((size_t)b * plane + (size_t)ys[a] * pw + xs[c]) * COUT + 32 * h);
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) p[u] = src[u];
-                        }
+                // stores of whole 64-byte runs: with each thread writing its own pixel
+                // the layer 16 -> 64 was bound by store wavefronts (256 x 256 x 64
+                // fields: 240 us, now 160; the hidden layers 281, now 271)
+                tc::store_row32<COUT>(aout, out, b, y, x0 + 32 * q, ny, nx, 32 * h);
             }
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
             __syncwarp();

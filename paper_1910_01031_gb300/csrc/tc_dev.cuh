@@ -172,6 +172,59 @@ __device__ __forceinline__ void stage_weights(unsigned char* wsm, const void* __
     }
 }
 
+// 4 x 4 transpose of 16-byte chunks over the four lanes 4 i .. 4 i + 3: lane l
+// gives chunks 0 .. 3 of its pixel and gets chunk l % 4 of the group's four
+// pixels.  A thread's 64 bytes of one pixel go to memory as four 16-byte
+// stores a pixel apart; after the transpose the four lanes of a store write
+// the 64 contiguous bytes of one pixel, a quarter of the lines per store and
+// whole sectors.
+__device__ __forceinline__ void transpose4(uint4 (&c)[4])
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int b = 1; b <= 2; b <<= 1) {
+        const bool hi = lane & b;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (u & b) continue;
+            uint32_t* lo_ = reinterpret_cast<uint32_t*>(&c[u]);
+            uint32_t* hi_ = reinterpret_cast<uint32_t*>(&c[u | b]);
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                const uint32_t got = __shfl_xor_sync(0xffffffffu, hi ? lo_[w] : hi_[w], b);
+                if (hi) lo_[w] = got;
+                else hi_[w] = got;
+            }
+        }
+    }
+}
+
+// 64 bytes per lane (32 BF16 channels from c0) of the pixels x .. of row y of
+// field b (lane l: pixel xw + l) into the padded [b][ny + 2][nx + 2][C] array
+// at the pixels and at their periodic halo images
+template <int C>
+__device__ __forceinline__ void store_row32(void* __restrict__ out, uint4 (&v)[4], int b, int y, int xw, int ny, int nx,
+                                            int c0)
+{
+    transpose4(v);
+    const int lane = threadIdx.x & 31;
+    const size_t pw = (size_t)(nx + 2), plane = (size_t)(ny + 2) * pw;
+    unsigned char* const o = static_cast<unsigned char*>(out) + (size_t)b * plane * (2 * C) + 2 * c0 + 16 * (lane & 3);
+    const int ys[2] = {y + 1, y == 0 ? ny + 1 : (y == ny - 1 ? 0 : -1)};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int x = xw + (lane & ~3) + u;
+        const int xs = x == 0 ? nx + 1 : (x == nx - 1 ? 0 : -1);
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+            if (ys[a] >= 0) {
+                unsigned char* const row = o + (size_t)ys[a] * pw * (2 * C);
+                *reinterpret_cast<uint4*>(row + (size_t)(x + 1) * (2 * C)) = v[u];
+                if (xs >= 0) *reinterpret_cast<uint4*>(row + (size_t)xs * (2 * C)) = v[u];
+            }
+    }
+}
+
 __device__ __forceinline__ void mma_commit(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar)
