@@ -171,8 +171,14 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmap_in, const __nv_bfloat16*
         __syncwarp();
     } else if (warp == 1) {
         // ---- MMA issuer ----
+        // the elected lane issues all products of a tile (its branch keeps the
+        // operands in uniform registers) and steps the descriptors by their
+        // lower words: with 64-bit steps in a lane == 0 branch a product took
+        // 100 cycles to issue and the tensor pipe waited (hidden layers, 256 x 256
+        // x 64 fields: 271 us, now 214 at 70% of the pipe; the last layer 225,
+        // now 146).  DRAM moves their 1.05 GB in 160 us
         int issued = 0;
-        if (lane == 0) {
+        if (tc::elect_one()) {
             constexpr uint32_t IDESC = idesc_bf16(TC_PX, COUT);
             for (int i = 0; i < nloc; ++i) {
                 const int s = i & 1;
@@ -185,9 +191,11 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmap_in, const __nv_bfloat16*
                 // descriptors of the stage and of the weights; every MMA adds a
                 // compile-time offset (in 16-byte units) to the address field
                 constexpr uint32_t PLANE = TC_PROWS * TC_PCOLS * 16;
-                const uint64_t adesc = L::SW ? sdesc(a0, 16, 1024, 2) : sdesc(a0, PLANE, 128, 0);
-                const uint64_t bdesc = L::SW ? sdesc(sbase + L::W_OFF, 16, 1024, 2)
-                                             : sdesc(sbase + L::W_OFF, COUT * 16, 128, 0);
+                const uint32_t adesc = (uint32_t)(L::SW ? sdesc(a0, 16, 1024, 2) : sdesc(a0, PLANE, 128, 0));
+                const uint32_t bdesc = (uint32_t)(L::SW ? sdesc(sbase + L::W_OFF, 16, 1024, 2)
+                                                        : sdesc(sbase + L::W_OFF, COUT * 16, 128, 0));
+                constexpr uint32_t AHI = (uint32_t)((L::SW ? sdesc(0, 16, 1024, 2) : sdesc(0, PLANE, 128, 0)) >> 32);
+                constexpr uint32_t BHI = (uint32_t)((L::SW ? sdesc(0, 16, 1024, 2) : sdesc(0, COUT * 16, 128, 0)) >> 32);
                 if constexpr (L::SW) {
                     // patch row p feeds output row r at ky = p - r; rows 1 and 2 feed
                     // both output rows at the same pixel alignment, so each is one
@@ -205,10 +213,10 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmap_in, const __nv_bfloat16*
                             auto boff = [&](int ky_top) {
                                 return (uint32_t)((((kx * 3 + 2 - ky_top) * COUT) * 128 + kc * 32) >> 4);
                             };
-                            tc::mma_bf16_ss(d0, adesc + aoff(1), bdesc + boff(1), ID2, (kx | kc) != 0);
-                            tc::mma_bf16_ss(d0, adesc + aoff(0), bdesc + boff(0), ID1, 1);
-                            tc::mma_bf16_ss(d0, adesc + aoff(2), bdesc + boff(2), ID2, 1);
-                            tc::mma_bf16_ss(d0 + (uint32_t)COUT, adesc + aoff(3), bdesc + boff(2), ID1, 1);
+                            tc::mma_bf16_lo(d0, adesc + aoff(1), AHI, bdesc + boff(1), BHI, ID2, (kx | kc) != 0);
+                            tc::mma_bf16_lo(d0, adesc + aoff(0), AHI, bdesc + boff(0), BHI, ID1, 1);
+                            tc::mma_bf16_lo(d0, adesc + aoff(2), AHI, bdesc + boff(2), BHI, ID2, 1);
+                            tc::mma_bf16_lo(d0 + (uint32_t)COUT, adesc + aoff(3), AHI, bdesc + boff(2), BHI, ID1, 1);
                         }
                 } else {
 #pragma unroll
@@ -222,14 +230,8 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmap_in, const __nv_bfloat16*
                                                         : (2 * kc * PLANE + ((r + ky) * TC_PCOLS + kx) * 16) >> 4;
                             const uint32_t boff = L::SW ? (tap * COUT * 128 + kc * 32) >> 4
                                                         : ((tap * (CIN / 8) + 2 * kc) * COUT * 16) >> 4;
-                            if ((tap | kc) != 0)
-                                asm volatile("tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, 1;\n" ::"r"(
-                                                 d0 + (uint32_t)(r * COUT)),
-                                             "l"(adesc + aoff), "l"(bdesc + boff), "r"(IDESC));
-                            else
-                                asm volatile("tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, 0;\n" ::"r"(
-                                                 d0 + (uint32_t)(r * COUT)),
-                                             "l"(adesc + aoff), "l"(bdesc + boff), "r"(IDESC));
+                            tc::mma_bf16_lo(d0 + (uint32_t)(r * COUT), adesc + aoff, AHI, bdesc + boff, BHI, IDESC,
+                                            (tap | kc) != 0);
                         }
                     }
                 }
@@ -289,7 +291,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmap_in, const __nv_bfloat16*
                 }
                 // stores of whole 64-byte runs: with each thread writing its own pixel
                 // the layer 16 -> 64 was bound by store wavefronts (256 x 256 x 64
-                // fields: 240 us, now 160; the hidden layers 281, now 271)
+                // fields: 240 us, now 160; the hidden layers 281 to 271)
                 tc::store_row32<COUT>(aout, out, b, y, x0 + 32 * q, ny, nx, 32 * h);
             }
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");

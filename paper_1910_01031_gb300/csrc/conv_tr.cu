@@ -50,7 +50,7 @@ namespace {
 using tc::idesc_bf16;
 using tc::mbar_drain;
 using tc::mbar_wait;
-using tc::mma_bf16_ss;
+using tc::mma_bf16_lo;
 using tc::mma_commit;
 using tc::sdesc;
 using tc::su32;
@@ -199,9 +199,12 @@ conv_tr_kernel(const __grid_constant__ CUtensorMap tmap_in, const __nv_bfloat16*
     } else if (warp == 1) {
         // ---- MMA issuer: 9 taps x CIN / 16 products of 128 x COUT x 16 per tile ----
         int committed = 0;
-        if (lane == 0) {
+        if (tc::elect_one()) {
             constexpr uint32_t IDESC = idesc_bf16(128, COUT);
-            const uint64_t bdesc = L::SW ? sdesc(sbase, 16, 1024, 2) : sdesc(sbase, COUT * 16, 128, 0);
+            const uint32_t bdesc = (uint32_t)(L::SW ? sdesc(sbase, 16, 1024, 2) : sdesc(sbase, COUT * 16, 128, 0));
+            constexpr uint32_t AHI =
+                (uint32_t)((L::SW ? sdesc(0, 16, TR_PW * 128, 2) : sdesc(0, L::PLANE, TR_PW * 16, 0)) >> 32);
+            constexpr uint32_t BHI = (uint32_t)((L::SW ? sdesc(0, 16, 1024, 2) : sdesc(0, COUT * 16, 128, 0)) >> 32);
             for (int i = 0; i < nloc; ++i) {
                 const int s = i % TR_NS, as = i & 1;
                 if (!mbar_wait(tempty0 + 8 * as, (uint32_t)(((i >> 1) & 1) ^ 1), abort)) break;
@@ -210,7 +213,8 @@ conv_tr_kernel(const __grid_constant__ CUtensorMap tmap_in, const __nv_bfloat16*
                 const uint32_t a0 = sbase + L::A_OFF + s * L::STAGE_ALLOC;
                 // A: the tile's 128 pixels as 16 rows of 8, one 8-row atom (or core
                 // matrix) per tile row, atoms one patch row (TR_PW pixels) apart
-                const uint64_t adesc = L::SW ? sdesc(a0, 16, TR_PW * 128, 2) : sdesc(a0, L::PLANE, TR_PW * 16, 0);
+                const uint32_t adesc =
+                    (uint32_t)(L::SW ? sdesc(a0, 16, TR_PW * 128, 2) : sdesc(a0, L::PLANE, TR_PW * 16, 0));
                 const uint32_t d0 = tmem + (uint32_t)(as * COUT);
 #pragma unroll
                 for (int tap = 0; tap < 9; ++tap) {
@@ -221,7 +225,7 @@ conv_tr_kernel(const __grid_constant__ CUtensorMap tmap_in, const __nv_bfloat16*
                                                     : (2 * kc * L::PLANE + (ky * TR_PW + kx) * 16) >> 4;
                         const uint32_t boff = L::SW ? (tap * COUT * 128 + kc * 32) >> 4
                                                     : ((tap * (CIN / 8) + 2 * kc) * COUT * 16) >> 4;
-                        mma_bf16_ss(d0, adesc + aoff, bdesc + boff, IDESC, (tap | kc) != 0);
+                        mma_bf16_lo(d0, adesc + aoff, AHI, bdesc + boff, BHI, IDESC, (tap | kc) != 0);
                     }
                 }
                 // the stage is free and the accumulator is ready once these products complete
@@ -423,8 +427,11 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         __syncwarp();
     } else if (warp == 1) {
         // ---- MMA issuer: 16 K steps of 16 pixels per tile, 5 tap pairs each ----
-        if (lane == 0) {
+        if (tc::elect_one()) {
             constexpr uint32_t IDESC = idesc_bf16(128, COUT, 1, 1);
+            constexpr uint32_t AHI = (uint32_t)(sdesc(0, 0, 1024, 2) >> 32);
+            constexpr uint32_t BHI =
+                (uint32_t)((COUT == 64 ? sdesc(0, 0, 1024, 2) : sdesc(0, 128, L::DPLANE, 0)) >> 32);
             for (int i = 0; i < nloc; ++i) {
                 const int s = i % WG_NS;
                 if (!mbar_wait(full0 + 8 * s, (uint32_t)((i / WG_NS) & 1), abort)) break;
@@ -434,8 +441,9 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
                 for (int st = 0; st < WG_ROWS * WG_PX / 16; ++st) {
                     const int r = st >> 2, xo = (st & 3) * 16;
                     // B = dZ^T (N = COUT channels, K = 16 pixels), M/N-major
-                    const uint64_t bdesc = COUT == 64 ? sdesc(ds + (uint32_t)((r * WG_PX + xo) * 128), 0, 1024, 2)
-                                                      : sdesc(ds + (uint32_t)((r * WG_PX + xo) * 16), 128, L::DPLANE, 0);
+                    const uint32_t bdesc =
+                        (uint32_t)(COUT == 64 ? sdesc(ds + (uint32_t)((r * WG_PX + xo) * 128), 0, 1024, 2)
+                                              : sdesc(ds + (uint32_t)((r * WG_PX + xo) * 16), 128, L::DPLANE, 0));
 #pragma unroll
                     for (int j = 0; j < WG_PAIRS; ++j) {
                         const int ta = wg_t0(j), tb = ta + 1;
@@ -445,8 +453,8 @@ wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
                         const uint32_t aaddr = j < WG_PAIRS - 1
                                                    ? xs + (uint32_t)(((r + ta / 3) * WG_PCOLS + xo + ta % 3) * 128)
                                                    : sbase;
-                        const uint64_t adesc = sdesc(aaddr, bstart - aaddr, 1024, 2);
-                        mma_bf16_ss(tmem + (uint32_t)(j * COUT), adesc, bdesc, IDESC, (i | st) != 0);
+                        const uint32_t adesc = (uint32_t)sdesc(aaddr, bstart - aaddr, 1024, 2);
+                        mma_bf16_lo(tmem + (uint32_t)(j * COUT), adesc, AHI, bdesc, BHI, IDESC, (i | st) != 0);
                     }
                 }
                 mma_commit(empty0 + 8 * s);

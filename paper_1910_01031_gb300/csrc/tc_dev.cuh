@@ -56,7 +56,7 @@ __device__ __forceinline__ uint32_t su32(const void* p)
 // swizzle) blocks along M/N and sbo = bytes between 8-row groups along K; no
 // swizzle, lbo = bytes between 8-row groups along K and sbo = bytes between
 // 8-element core matrices along M/N.
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t sbo, uint32_t layout)
+__host__ __device__ constexpr uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t sbo, uint32_t layout)
 {
     return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
            ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46) | ((uint64_t)(layout & 7) << 61);
@@ -130,14 +130,32 @@ __device__ __forceinline__ void tmem_ld32(uint32_t ta, uint32_t* r)
     asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 }
 
-__device__ __forceinline__ void mma_bf16_ss(uint32_t d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, int acc)
+// true in one lane of a converged warp; the compiler knows that a branch on it
+// has one active lane, and keeps what is computed there in uniform registers
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t e;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+    return e != 0;
+}
+
+// D (+)= A B with the operands' descriptors given as their constant upper word
+// and their lower word (start address and leading stride).  A step through the
+// operand is an addition to the lower word alone: the upper words, the
+// accumulator and the instruction descriptor stay in uniform registers over a
+// whole tile, where 64-bit descriptors are moved there word by word before
+// every product
+__device__ __forceinline__ void mma_bf16_lo(uint32_t d, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
+                                            uint32_t idesc, int acc)
 {
     if (acc)
-        asm volatile("tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, 1;\n" ::"r"(d), "l"(adesc), "l"(bdesc),
-                     "r"(idesc));
+        asm volatile("{\n .reg .b64 a, b;\n mov.b64 a, {%1, %2};\n mov.b64 b, {%3, %4};\n"
+                     " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, 1;\n}\n" ::"r"(d),
+                     "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc));
     else
-        asm volatile("tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, 0;\n" ::"r"(d), "l"(adesc), "l"(bdesc),
-                     "r"(idesc));
+        asm volatile("{\n .reg .b64 a, b;\n mov.b64 a, {%1, %2};\n mov.b64 b, {%3, %4};\n"
+                     " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, 0;\n}\n" ::"r"(d),
+                     "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc));
 }
 
 // stage the weights of every tap once per CTA (B operand, K-major, rows =
