@@ -292,7 +292,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmap_in, const __nv_bfloat16*
                 // stores of whole 64-byte runs: with each thread writing its own pixel
                 // the layer 16 -> 64 was bound by store wavefronts (256 x 256 x 64
                 // fields: 240 us, now 160; the hidden layers 281 to 271)
-                tc::store_row32<COUT>(aout, out, b, y, x0 + 32 * q, ny, nx, 32 * h);
+                tc::store_padded32<COUT>(aout, out, b, y, x, ny, nx, 32 * h);
             }
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
             __syncwarp();

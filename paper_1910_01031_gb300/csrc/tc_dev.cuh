@@ -217,30 +217,52 @@ __device__ __forceinline__ void transpose4(uint4 (&c)[4])
     }
 }
 
-// 64 bytes per lane (32 BF16 channels from c0) of the pixels x .. of row y of
-// field b (lane l: pixel xw + l) into the padded [b][ny + 2][nx + 2][C] array
-// at the pixels and at their periodic halo images
+// 64 bytes per lane (32 BF16 channels from c0) of pixel x of row y of field b
+// (four neighbouring lanes: four neighbouring pixels from a multiple of 4)
+// into the padded [b][ny + 2][nx + 2][C] array at the pixel and at its
+// periodic halo images
 template <int C>
-__device__ __forceinline__ void store_row32(void* __restrict__ out, uint4 (&v)[4], int b, int y, int xw, int ny, int nx,
-                                            int c0)
+__device__ __forceinline__ void store_padded32(void* __restrict__ out, uint4 (&v)[4], int b, int y, int x, int ny,
+                                               int nx, int c0)
 {
     transpose4(v);
-    const int lane = threadIdx.x & 31;
+    const int l4 = threadIdx.x & 3;
     const size_t pw = (size_t)(nx + 2), plane = (size_t)(ny + 2) * pw;
-    unsigned char* const o = static_cast<unsigned char*>(out) + (size_t)b * plane * (2 * C) + 2 * c0 + 16 * (lane & 3);
+    unsigned char* const o = static_cast<unsigned char*>(out) + (size_t)b * plane * (2 * C) + 2 * c0 + 16 * l4;
     const int ys[2] = {y + 1, y == 0 ? ny + 1 : (y == ny - 1 ? 0 : -1)};
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-        const int x = xw + (lane & ~3) + u;
-        const int xs = x == 0 ? nx + 1 : (x == nx - 1 ? 0 : -1);
+        const int xu = x - l4 + u;
+        const int xs = xu == 0 ? nx + 1 : (xu == nx - 1 ? 0 : -1);
 #pragma unroll
         for (int a = 0; a < 2; ++a)
             if (ys[a] >= 0) {
                 unsigned char* const row = o + (size_t)ys[a] * pw * (2 * C);
-                *reinterpret_cast<uint4*>(row + (size_t)(x + 1) * (2 * C)) = v[u];
+                *reinterpret_cast<uint4*>(row + (size_t)(xu + 1) * (2 * C)) = v[u];
                 if (xs >= 0) *reinterpret_cast<uint4*>(row + (size_t)xs * (2 * C)) = v[u];
             }
     }
+}
+
+// the same four lanes' 64 bytes per pixel of an unpadded row of C-channel
+// pixels; p is the address of channel 0 of the lane's own pixel
+template <int C>
+__device__ __forceinline__ void store_pixels32(void* __restrict__ p, uint4 (&v)[4], int c0)
+{
+    transpose4(v);
+    const int l4 = threadIdx.x & 3;
+    unsigned char* const o = static_cast<unsigned char*>(p) - l4 * (2 * C) + 2 * c0 + 16 * l4;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) *reinterpret_cast<uint4*>(o + u * (2 * C)) = v[u];
+}
+template <int C>
+__device__ __forceinline__ void load_pixels32(const void* __restrict__ p, uint4 (&v)[4], int c0)
+{
+    const int l4 = threadIdx.x & 3;
+    const unsigned char* const o = static_cast<const unsigned char*>(p) - l4 * (2 * C) + 2 * c0 + 16 * l4;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = *reinterpret_cast<const uint4*>(o + u * (2 * C));
+    transpose4(v);
 }
 
 __device__ __forceinline__ void mma_commit(uint32_t bar)
