@@ -1,13 +1,18 @@
 // IEWPF analysis kernels for one problem per launch (Sec. 4 and App. A of
 // arXiv 1910.01031); the device code is in analysis_dev.cuh.
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "analysis_dev.cuh"
+#include "tc_dev.cuh"
 
 namespace iewpf {
 
 namespace {
+
+// dynamic shared memory of a CTA of the grouped sweeps at most
+constexpr int kSolveGroupSmem = 224 * 1024;
 
 __global__ void obs_cells_kernel(const double* __restrict__ xy, int nobs, Grid G, Coarse C, double dx, double dy,
                                  int* __restrict__ cell, int* __restrict__ block0)
@@ -100,6 +105,52 @@ solve_smem_kernel(const double* __restrict__ L, const int* __restrict__ colptr, 
 {
     extern __shared__ double sx[];
     ana::solve_levels_warp(L, colptr, rowidx, rdiag, plan, n, d, x, phi, blockIdx.x, perm, nullptr, Lr, Lc, sx);
+}
+
+// the factor in the order of the sweeps: rows, diagonals and steps of both
+// directions (a warp each), then the entries (a warp per position)
+__global__ void __launch_bounds__(32)
+sweep_rows_kernel(const int* plan, int n, int nnz, const double* __restrict__ rdiag, void* stream)
+{
+    const ana::SolvePlan P = ana::solve_plan_view(const_cast<int*>(plan), n);
+    const bool back = blockIdx.x;
+    const ana::SweepStream S =
+        ana::sweep_stream_view(static_cast<char*>(stream) + back * ana::sweep_stream_bytes(n, nnz), n, nnz);
+    ana::sweep_rows_warp(back ? P.rb : P.rf, back ? P.bptr : P.fptr, P.nlev[back], n, rdiag, S);
+}
+__global__ void sweep_entries_kernel(const double* __restrict__ L, const int* plan, int n, int nnz,
+                                     const int* __restrict__ rowidx, void* stream)
+{
+    const ana::SolvePlan P = ana::solve_plan_view(const_cast<int*>(plan), n);
+    const bool back = blockIdx.y;
+    const ana::SweepStream S =
+        ana::sweep_stream_view(static_cast<char*>(stream) + back * ana::sweep_stream_bytes(n, nnz), n, nnz);
+    const int lane = threadIdx.x & 31;
+    for (int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < n; t += (gridDim.x * blockDim.x) >> 5) {
+        const int4 r = S.row[t];
+        const int q0 = (back ? P.rb : P.rf)[3 * t + 1];
+        for (int q = lane; q < r.z - r.y; q += 32) {
+            const int j = (back ? rowidx : P.colidx)[q0 + q];
+            S.ent[r.y + q] = {back ? L[(long long)j * n + r.x] : L[(long long)r.x * n + j], j, 0};
+        }
+    }
+}
+
+// P particles per CTA.  The sweeps are a chain of levels (2 x 544 for 1521
+// coupled moorings), each a barrier and the FP64 latency of its longest sum;
+// the warp per particle of solve_smem_kernel also waited on L2 for every
+// level's entries, which it read for that particle alone (1000 particles: 5.5
+// ms, now 3.4; FP64 pipe active half of the time)
+template <int P>
+__global__ void __launch_bounds__(32 * P)
+solve_group_kernel(const void* stream, int n, int nnz, const double* __restrict__ d, double* __restrict__ x,
+                   double* __restrict__ phi, int ne, const int* __restrict__ perm)
+{
+    extern __shared__ __align__(16) double group_smem[];
+    char* base = static_cast<char*>(const_cast<void*>(stream));
+    ana::solve_group_cta<P>(ana::sweep_stream_view(base, n, nnz),
+                            ana::sweep_stream_view(base + ana::sweep_stream_bytes(n, nnz), n, nnz), n, nnz, d, x, phi,
+                            blockIdx.x * P, ne, perm, group_smem);
 }
 
 __global__ void __launch_bounds__(ana::DOT_THREADS)
@@ -269,10 +320,35 @@ cudaError_t launch_cholesky(double* M, int n, int* colptr, int* rowidx, int* fla
 
 cudaError_t launch_solve(const double* L, const int* colptr, const int* rowidx, const double* rdiag, const int* plan,
                          int n, const double* d, double* Sd, double* phi, int ne, cudaStream_t st, const int* perm,
-                         double* scratch, const double* Lr, const double* Lc)
+                         double* scratch, const double* Lr, const double* Lc, const void* stream, int nnz)
 {
     if ((perm && !scratch) || (!Lr != !Lc)) return cudaErrorInvalidValue;
     if (ne <= 0) return cudaSuccess;
+    // Several particles per CTA where that takes at most 3 / 2 as many waves of
+    // CTAs as a warp each does (a wave of 1521 coupled moorings, n = 3042: 3.4 ms
+    // against 5.5), and of 4 and 8 the one with fewer waves (4 at a tie: 5350
+    // against 5624 us per analysis of 100 particles; of 1000, 8 takes one wave
+    // and 13.2 ms, 4 two and 16.0, a warp each 15.4)
+    if (stream && n > 0) {
+        const int sms = tc::sm_count();
+        auto waves = [&](int P, size_t smem) {
+            const size_t resident = std::min((size_t)16 / P, (size_t)(228 * 1024) / (smem + 1024));
+            return resident ? ((size_t)(ne + P - 1) / P + sms * resident - 1) / (sms * resident) : (size_t)1 << 30;
+        };
+        auto group_waves = [&](int P, size_t smem) { return smem <= kSolveGroupSmem ? waves(P, smem) : (size_t)1 << 30; };
+        const size_t w1 = waves(1, (size_t)n * sizeof(double)), w4 = group_waves(4, ana::solve_group_smem<4>(n)),
+                     w8 = group_waves(8, ana::solve_group_smem<8>(n));
+        auto group = [&](auto Pc) {
+            constexpr int P = decltype(Pc)::value;
+            cudaError_t e = tc::smem_attr_once<solve_group_kernel<P>>(kSolveGroupSmem);
+            if (e != cudaSuccess) return e;
+            solve_group_kernel<P><<<(ne + P - 1) / P, 32 * P, ana::solve_group_smem<P>(n), st>>>(stream, n, nnz, d, Sd,
+                                                                                                phi, ne, perm);
+            return cudaGetLastError();
+        };
+        if (2 * std::min(w4, w8) <= 3 * w1)
+            return w4 <= w8 ? group(std::integral_constant<int, 4>()) : group(std::integral_constant<int, 8>());
+    }
     if (n > 0 && (size_t)n * sizeof(double) <= kSolveSmemBytes) {
         solve_smem_kernel<<<ne, 32, (size_t)n * sizeof(double), st>>>(L, colptr, rowidx, rdiag, plan, n, d, Sd, phi,
                                                                        perm, Lr, Lc);
@@ -292,6 +368,19 @@ cudaError_t launch_pack_factor(const double* L, int n, const int* colptr, const 
     const int threads = 256;
     const int blocks = std::min((n * 32 + threads - 1) / threads, 65535);
     pack_factor_kernel<<<blocks, threads, 0, st>>>(L, n, colptr, rowidx, plan, Lr, Lc);
+    return cudaGetLastError();
+}
+
+size_t solve_stream_bytes(int n, int nnz) { return 2 * ana::sweep_stream_bytes(n, nnz); }
+
+cudaError_t launch_pack_stream(const double* L, int n, int nnz, const int* rowidx, const int* plan, const double* rdiag,
+                               void* stream, cudaStream_t st)
+{
+    if (n <= 0) return cudaSuccess;
+    sweep_rows_kernel<<<2, 32, 0, st>>>(plan, n, nnz, rdiag, stream);
+    const int threads = 256;
+    const dim3 blocks(std::min((n * 32 + threads - 1) / threads, 65535), 2);
+    sweep_entries_kernel<<<blocks, threads, 0, st>>>(L, plan, n, nnz, rowidx, stream);
     return cudaGetLastError();
 }
 

@@ -489,6 +489,275 @@ __device__ __forceinline__ void solve_levels_warp(const double* __restrict__ L, 
     }
 }
 
+// The factor as the two sweeps read it, for solve_group_cta: positions t of the
+// level order hold row[t] = {row (column) i, first entry, end, -} and its
+// reciprocal diagonal rd[t]; the entries (in the order of the CSR or CSC) are
+// contiguous along the order.  step[s] = {first position, rows (at most 32) +
+// 256 log2 of the lanes per row, first entry, end}: a level, or a round of 32
+// rows of a wider one.
+struct __align__(16) SweepEntry {
+    double val;
+    int idx, pad;
+};
+struct SweepStream {
+    int4 *step, *row;   // [n] each
+    SweepEntry* ent;    // [nnz]
+    double* rd;         // [n]
+    int* nstep;         // [1]
+};
+// bytes of one direction's arrays, and its view at base (16-byte aligned)
+__host__ __device__ __forceinline__ size_t sweep_stream_bytes(int n, int nnz)
+{
+    return 16 * (2 * (size_t)n + nnz + ((size_t)n + 1) / 2 + 1);
+}
+__host__ __device__ __forceinline__ SweepStream sweep_stream_view(void* base, int n, int nnz)
+{
+    SweepStream S;
+    S.step = static_cast<int4*>(base);
+    S.row = S.step + n;
+    S.ent = reinterpret_cast<SweepEntry*>(S.row + n);
+    S.nstep = reinterpret_cast<int*>(S.ent + nnz);
+    S.rd = reinterpret_cast<double*>(S.ent + nnz + 1);
+    return S;
+}
+
+// warp: row, rd and the steps of one direction from the plan's triples ri and
+// level bounds lv[0..nl]
+__device__ __forceinline__ void sweep_rows_warp(const int* __restrict__ ri, const int* __restrict__ lv, int nl, int n,
+                                                const double* __restrict__ rdiag, const SweepStream& S)
+{
+    const int lane = threadIdx.x & 31;
+    int base = 0;
+    for (int t0 = 0; t0 < n; t0 += 32) {
+        const int t = t0 + lane;
+        const int len = t < n ? ri[3 * t + 2] - ri[3 * t + 1] : 0;
+        int end = len;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, end, o);
+            if (lane >= o) end += v;
+        }
+        if (t < n) {
+            S.row[t] = make_int4(ri[3 * t], base + end - len, base + end, 0);
+            S.rd[t] = rdiag[ri[3 * t]];
+        }
+        base += __shfl_sync(0xffffffffu, end, 31);
+    }
+    __syncwarp();
+    int ns = 0;
+    if (lane == 0) {
+        for (int l = 0; l < nl; ++l) {
+            const int m = lv[l + 1] - lv[l];
+            const int lg = m >= 32 ? 0 : 5 - (m <= 1 ? 0 : 32 - __clz(m - 1));
+            for (int t = lv[l]; t < lv[l + 1]; t += 32) {
+                const int e = min(t + 32, lv[l + 1]);
+                S.step[ns++] = make_int4(t, (e - t) + 256 * lg, S.row[t].y, S.row[e - 1].z);
+            }
+        }
+        *S.nstep = ns;
+    }
+}
+
+__device__ __forceinline__ void cp_async16(void* s, const void* g)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((uint32_t)__cvta_generic_to_shared(s)), "l"(g)
+                 : "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
+
+// CTA of 32 P threads: solve_levels_warp for P particles together, their
+// vectors interleaved in shared memory (entry i of particle p at i P + p).  The
+// 32 lanes that a level's rows share there are 32 slots here, of P lanes each,
+// one per particle: a factor entry is loaded once for P particles, and the
+// slots spread over P warps.  The entries flow through a ring in shared memory
+// (cp.async, several steps ahead), so that a step waits on shared memory and
+// its FP64 chain alone.  A row's partial sums, their order and the order of the
+// group's sum are those of solve_levels_warp: the same bits.
+constexpr int SOLVE_RING = 2048;      // entries
+template <int P>
+__host__ __device__ constexpr size_t solve_group_smem(int n)
+{
+    return SOLVE_RING * sizeof(SweepEntry) + ((size_t)n * P + P * P) * sizeof(double);
+}
+template <int P>
+__device__ __forceinline__ void solve_group_cta(const SweepStream& F, const SweepStream& B, int n, int nnz,
+                                                const double* __restrict__ d, double* __restrict__ x,
+                                                double* __restrict__ phi, int w0, int ne,
+                                                const int* __restrict__ perm, double* smem)
+{
+    constexpr int S = 32 / P;      // slots per warp (P warps)
+    constexpr int LS = P == 4 ? 3 : 2;
+    static_assert(1 << LS == S, "slots per warp");
+    SweepEntry* const rent = reinterpret_cast<SweepEntry*>(smem);
+    double* const part = smem + SOLVE_RING * (sizeof(SweepEntry) / sizeof(double));
+    double* const sx = part + P * P;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int p = lane % P, slot = lane / P;
+    const int np = min(P, ne - w0);
+    for (int k = tid; k < n * np; k += 32 * P) {
+        const int w = k / n, i = k - w * n;
+        sx[i * P + w] = d[(long long)(w0 + w) * n + (perm ? perm[i] : i)];
+    }
+    if (np < P)
+        for (int k = tid; k < n; k += 32 * P)
+            for (int w = np; w < P; ++w) sx[k * P + w] = 0.0;
+    auto sweep = [&](const SweepStream& Q) {
+        const int ns = *Q.nstep;
+        int issued = 0;
+        auto top_up = [&](int upto) {
+            for (int q = issued + tid; q < upto; q += 32 * P) {
+                cp_async16(rent + (q & (SOLVE_RING - 1)), Q.ent + q);
+            }
+            issued = max(issued, upto);
+            asm volatile("cp.async.commit_group;\n" ::: "memory");
+        };
+        auto step_at = [&](int k) { return k < ns ? Q.step[k] : make_int4(n, 0, nnz, nnz); };
+        // this slot's row of a step {row (-1: none), first entry, end, diagonal} and
+        // place in the row's group of g slots: the upper bits of the place are the
+        // slot's in its warp, so that the halves that the group's sum joins first
+        // lie in one warp
+        struct Row {
+            int i, q0, q1;
+            double rd;
+        };
+        auto row_at = [&](const int4& st) {
+            const int lg = st.y >> 8, m = st.y & 255;
+            int r, sub;
+            if (lg >= LS) {
+                r = warp >> (lg - LS);
+                sub = (warp & ((1 << (lg - LS)) - 1)) + (slot << (lg - LS));
+            } else {
+                r = (warp << (LS - lg)) + (slot >> lg);
+                sub = slot & ((1 << lg) - 1);
+            }
+            Row R{-1, 0, 0, 0.0};
+            if (r < m) {
+                const int4 v = Q.row[st.x + r];
+                R.i = v.x;
+                R.q0 = v.y + sub;
+                R.q1 = v.z;
+                R.rd = Q.rd[st.x + r];
+            }
+            return R;
+        };
+        int4 s0 = step_at(0), s1 = step_at(1), s2 = step_at(2);
+        Row r0 = row_at(s0), r1 = row_at(s1);
+        top_up(min(nnz, SOLVE_RING));
+        cp_async_wait<0>();
+        __syncthreads();
+        int safe = issued, mark1 = issued, mark2 = issued;   // entries arrived; issued one and two steps ago
+#pragma unroll 3
+        for (int k = 0; k < ns; ++k) {
+            const int4 s3 = step_at(k + 3);
+            const Row r2 = row_at(s2);
+            // what precedes this step's entries is free
+            issued = max(issued, s0.z);
+            top_up(min(nnz, s0.z + SOLVE_RING));
+            const bool ring = s0.w - s0.z <= SOLVE_RING;
+            if (ring && s0.w > safe) {
+                cp_async_wait<0>();
+                __syncthreads();
+                safe = issued;
+            }
+            const int lg = s0.y >> 8, g = 1 << lg;
+            double acc = 0.0;
+            // batches of 8 entries, a last one of those that are left
+            auto products = [&](const SweepEntry* ent, int mask) {
+                constexpr int U = 8;
+                int q = r0.q0, left = (r0.q1 - r0.q0 + g - 1) >> lg;
+                for (; left >= U; left -= U, q += U << lg) {
+                    double v[U], xv[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const SweepEntry e = ent[(q + (u << lg)) & mask];
+                        v[u] = e.val;
+                        xv[u] = sx[e.idx * P + p];
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u) acc = fma(v[u], xv[u], acc);
+                }
+                if (left > 0) {
+                    double v[U - 1], xv[U - 1];
+#pragma unroll
+                    for (int u = 0; u < U - 1; ++u)
+                        if (u < left) {
+                            const SweepEntry e = ent[(q + (u << lg)) & mask];
+                            v[u] = e.val;
+                            xv[u] = sx[e.idx * P + p];
+                        }
+#pragma unroll
+                    for (int u = 0; u < U - 1; ++u)
+                        if (u < left) acc = fma(v[u], xv[u], acc);
+                }
+            };
+            if (ring) products(rent, SOLVE_RING - 1);
+            else products(Q.ent, -1);
+            __syncwarp();
+            for (int o = min(g, S) >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o * P);
+            if (g <= S) {
+                if (r0.i >= 0 && (slot & (g - 1)) == 0) sx[r0.i * P + p] = (sx[r0.i * P + p] - acc) * r0.rd;
+            } else {
+                // the group's sum over its warps
+                const int wg = 1 << (lg - LS);
+                if (slot == 0) part[warp * P + p] = acc;
+                __syncthreads();
+                if (r0.i >= 0 && slot == 0 && (warp & (wg - 1)) == 0) {
+                    double v[P];
+#pragma unroll
+                    for (int c = 0; c < P; ++c) v[c] = c < wg ? part[(warp + c) * P + p] : 0.0;
+#pragma unroll
+                    for (int o = P / 2; o > 0; o >>= 1)
+                        if (o < wg)
+#pragma unroll
+                            for (int c = 0; c < o; ++c) v[c] += v[c + o];
+                    sx[r0.i * P + p] = (sx[r0.i * P + p] - v[0]) * r0.rd;
+                }
+            }
+            // the next step's entries: the copies of this step and of the one
+            // before may stay in flight if none of them are among those (none do
+            // after a step too large for the ring, whose own copies nobody reads)
+            if (ring && s1.w <= mark2) {
+                cp_async_wait<2>();
+                safe = max(safe, mark2);
+            } else if (ring && s1.w <= mark1) {
+                cp_async_wait<1>();
+                safe = max(safe, mark1);
+            } else {
+                cp_async_wait<0>();
+                safe = issued;
+            }
+            __syncthreads();
+            mark2 = mark1;
+            mark1 = issued;
+            s0 = s1; s1 = s2; s2 = s3;
+            r0 = r1; r1 = r2;
+        }
+        cp_async_wait<0>();
+        __syncthreads();
+    };
+    __syncthreads();
+    sweep(F);
+    sweep(B);
+    // phi, a warp per particle, and the solution in the observations' order
+    if (warp < np) {
+        const double* dp = d + (long long)(w0 + warp) * n;
+        double* out = x + (long long)(w0 + warp) * n;
+        double acc = 0.0;
+        for (int i = lane; i < n; i += 32) {
+            const int o = perm ? perm[i] : i;
+            const double v = sx[i * P + warp];
+            acc = fma(dp[o], v, acc);
+            out[o] = v;
+        }
+        acc = warp_sum(acc);
+        if (lane == 0) phi[w0 + warp] = acc;
+    }
+}
+
 constexpr int DOT_THREADS = 256;
 constexpr int DOT_BLOCKS_PER_CTA = 8;
 

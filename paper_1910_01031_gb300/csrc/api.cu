@@ -105,6 +105,8 @@ struct iewpf_ctx {
     // plan's rows and of the CSC (launch_pack_factor); null for drifters
     double* d_Lr = nullptr;
     double* d_Lc = nullptr;
+    char* d_stream = nullptr;     // the same in the order of the sweeps (launch_pack_stream)
+    int nnz = 0;
     double* d_d = nullptr;      // innovations [ne][Ny]
     double* d_Sd = nullptr;     // [ne][Ny]
     double* d_phi = nullptr;
@@ -946,6 +948,14 @@ int iewpf_create(const iewpf_params_t* params, const double* mooring_xy, iewpf_c
         if (cudaMemcpy(&nnz, ctx->d_colptr + 2 * nobs, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
             return bail(IEWPF_ECUDA);
         if ((rc = dalloc(ctx, &ctx->d_Lr, (size_t)nnz)) || (rc = dalloc(ctx, &ctx->d_Lc, (size_t)nnz))) return bail(rc);
+        ctx->nnz = nnz;
+        // (121 coupled moorings: 1031 us per analysis of 40 particles with a warp per
+        // particle, 1053 with the stream; 1024 of them and 100 particles: 3553 and 2768)
+        if (nobs >= kNdMinObs &&
+            ((rc = dalloc(ctx, &ctx->d_stream, solve_stream_bytes(2 * nobs, nnz))) ||
+             launch_pack_stream(ctx->d_L, 2 * nobs, nnz, ctx->d_rowidx, ctx->d_plan, ctx->d_rdiag, ctx->d_stream,
+                                ctx->st) != cudaSuccess))
+            return bail(rc ? rc : IEWPF_ECUDA);
         if (launch_pack_factor(ctx->d_L, 2 * nobs, ctx->d_colptr, ctx->d_rowidx, ctx->d_plan, ctx->d_Lr, ctx->d_Lc,
                                ctx->st) != cudaSuccess)
             return bail(IEWPF_ECUDA);
@@ -976,7 +986,7 @@ int iewpf_destroy(iewpf_ctx_t* ctx)
                     ctx->d_wtab, ctx->d_K32, ctx->d_K64, ctx->d_M49, ctx->d_xy, ctx->d_obs_xy, ctx->d_obs_y,
                     ctx->d_cell, ctx->d_block0, ctx->d_border, ctx->d_blevel, ctx->d_perm_u, ctx->d_cell_perm, ctx->d_xs,
                     ctx->d_tile_cnt, ctx->d_tile_obs, ctx->d_L, ctx->d_colptr,
-                    ctx->d_rowidx, ctx->d_rdiag, ctx->d_plan, ctx->d_Lr, ctx->d_Lc, ctx->d_d, ctx->d_Sd, ctx->d_phi, ctx->d_c, ctx->d_gamma, ctx->d_zeta,
+                    ctx->d_rowidx, ctx->d_rdiag, ctx->d_plan, ctx->d_Lr, ctx->d_Lc, ctx->d_stream, ctx->d_d, ctx->d_Sd, ctx->d_phi, ctx->d_c, ctx->d_gamma, ctx->d_zeta,
                     ctx->d_alpha, ctx->d_cstar, ctx->d_neglogw, ctx->d_coef, ctx->d_scal, ctx->d_partial,
                     ctx->d_r, ctx->d_xi, ctx->d_soar};
     for (void* p : ptrs)
@@ -1087,7 +1097,7 @@ int iewpf_assimilate(iewpf_ctx_t* ctx, const iewpf_obs_t* obs, iewpf_diag_t* dia
         if (!mooring && (rc = factor(ctx, nobs))) return rc;
         KL(1, launch_solve(ctx->d_L, ctx->d_colptr, ctx->d_rowidx, ctx->d_rdiag, ctx->d_plan, n, ctx->d_d, ctx->d_Sd,
                            ctx->d_phi, ne, ctx->st, ctx->d_perm_u, ctx->d_xs, mooring ? ctx->d_Lr : nullptr,
-                           mooring ? ctx->d_Lc : nullptr));
+                           mooring ? ctx->d_Lc : nullptr, mooring ? ctx->d_stream : nullptr, ctx->nnz));
     }
     // 3: random vectors
     Phase sub_("weights_and_update");

@@ -177,7 +177,12 @@ constexpr size_t kSolveSmemBytes = 48 * 1024;
 cudaError_t launch_solve(const double* L, const int* colptr, const int* rowidx, const double* rdiag, const int* plan,
                          int n, const double* d, double* Sd, double* phi, int ne, cudaStream_t st,
                          const int* perm = nullptr, double* scratch = nullptr, const double* Lr = nullptr,
-                         const double* Lc = nullptr);
+                         const double* Lc = nullptr, const void* stream = nullptr, int nnz = 0);
+// after launch_cholesky: the factor (nnz entries below the diagonal) in the
+// order of the sweeps, solve_stream_bytes(n, nnz) bytes
+size_t solve_stream_bytes(int n, int nnz);
+cudaError_t launch_pack_stream(const double* L, int n, int nnz, const int* rowidx, const int* plan, const double* rdiag,
+                               void* stream, cudaStream_t st);
 // after launch_cholesky: the factor's values below the diagonal in the order
 // of the plan's rows (Lr) and of the CSC (Lc), n (n - 1) / 2 doubles each at
 // most

@@ -133,3 +133,25 @@ def test_resident_model_steps_equal_the_march(nx, ny, c):
     assert np.array_equal(a.last_nsub(), b.last_nsub())
     assert a.work() - w0 == b.work()
     assert a.counters() == b.counters()
+
+
+@pytest.mark.parametrize("m,spacing,ne", [(16, 5, 1), (17, 5, 9), (17, 8, 6), (36, 5, 611)])
+def test_grouped_sweeps_equal_a_warp_per_particle(m, spacing, ne):
+    """Layouts of 256 moorings and more: the triangular sweeps of 4 or 8 particles per CTA (ragged last groups,
+    coupled and uncoupled factors) against the batch's, which take a warp per particle, bit for bit."""
+    n = 16 * (-(-(m * spacing + 8) // 16))
+    cfg = synth.Config("edge", n, n, n_particles=ne, n_obs=m * m, obs_kind=synth.OBS_MOORING, c_omega=1)
+    cells = np.array([[4 + spacing * (k % m), 3 + spacing * (k // m)] for k in range(m * m)])
+    xy = synth.cell_positions(cfg, cells)
+    batch = iewpf.Batch([iewpf.params_from_config(cfg)], [xy])
+    single = ensemble(cfg, mooring_xy=xy)
+    U = np.repeat(synth.initial_state(cfg, min(ne, 20), seed=7).astype(np.float32), -(-ne // 20), axis=0)[:ne]
+    y = synth.obs_from_state(cfg, synth.initial_particle(cfg, 77, seed=5), cells, synth.obs_noise(cfg, m * m, 0))
+    for e in (single, batch.instances[0]):
+        e.set_state(U)
+    diag = batch.cycle(2, [(None, y)])
+    single.forecast(1, True)
+    single.forecast(1, False)
+    d = single.assimilate(None, y)
+    assert diag[0, 0] == d["w_target"] and diag[0, 1] == d["beta"] and diag[0, 2] == 0
+    assert np.array_equal(batch.instances[0].get_state(), single.get_state())
