@@ -194,55 +194,53 @@ __global__ void form_r_kernel(uint64_t seed, uint32_t t, uint32_t s_xi, uint32_t
     if (4 * q < NR) ana::form_r_block(seed, t, s_xi, s_nu, NR, coef, scal, alpha, r, blockIdx.y, q);
 }
 
-__global__ void block_seq_kernel(float* __restrict__ r, int NR, const float* __restrict__ M49,
-                                 const int* __restrict__ block0, int nobs, int nRx, int nRy)
+// blocks that follow each other in every particle (positions that change each
+// cycle): a warp per particle; two barriers and a round trip per block before
+// (64 drifters x 100: 85 us, now 32)
+__global__ void __launch_bounds__(32)
+block_seq_kernel(float* __restrict__ r, int NR, const float* __restrict__ M49, const int* __restrict__ block0, int nobs,
+                 int nRx, int nRy)
 {
-    ana::block_seq_cta(r, NR, M49, block0, nobs, nRx, nRy, blockIdx.x);
+    __shared__ __align__(16) float v[3 * 52];
+    ana::block_seq_warp(r, NR, M49, block0, nobs, nRx, nRy, blockIdx.x, v);
 }
 
 // all levels of the local blocks of particle blockIdx.x: the CTA's warps
-// share the blocks of a level, a barrier separates the levels; lane t
-// computes outputs t and t + 32 (< 49) with the FMA order of block_seq_cta,
-// its two rows of the 49 x 49 root held in registers
-constexpr int BL_THREADS = 64;
-__global__ void __launch_bounds__(BL_THREADS) block_levels_kernel(float* __restrict__ r, int NR,
-                                                                  const float* __restrict__ M49,
-                                                                  const int* __restrict__ block0,
-                                                                  const int* __restrict__ order,
-                                                                  const int* __restrict__ level_off, int nlev,
-                                                                  int nRx, int nRy)
+// share the blocks of a level (cells: their places, level by level), a barrier
+// separates the levels.  Bound by latency: enough warps per particle to fill
+// the chip and the next block's inputs in flight (1521 blocks x 256 particles
+// on one level: 755 us with 2 warps, now 134)
+constexpr int BL_WARPS = 16;
+__global__ void __launch_bounds__(32 * BL_WARPS)
+block_levels_kernel(float* r, int NR, const float* __restrict__ M49, const int2* __restrict__ cells,
+                    const int* __restrict__ level_off, int nlev, int nRx, int nRy)
 {
-    __shared__ float v[BL_THREADS / 32][49];
-    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-    const bool two = lane + 32 < 49;
-    float m0[49], m1[49];
-#pragma unroll
-    for (int j = 0; j < 49; ++j) {
-        m0[j] = __ldg(M49 + lane * 49 + j);
-        m1[j] = two ? __ldg(M49 + (lane + 32) * 49 + j) : 0.0f;
-    }
+    __shared__ __align__(16) float v[BL_WARPS][52];
+    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    ana::BlockRoot M;
+    M.load(M49);
     float* rp = r + (long long)blockIdx.x * NR;
     for (int lev = 0; lev < nlev; ++lev) {
-        const int lo = level_off[lev], hi = level_off[lev + 1];
-        for (int ib = lo + wl; ib < hi; ib += BL_THREADS / 32) {
-            const int l = order[ib];
-            const int cx = block0[2 * l], cy = block0[2 * l + 1];
-            const int i0 = pmod(cy + lane / 7 - 3, nRy) * nRx + pmod(cx + lane % 7 - 3, nRx);
-            const int t1 = two ? lane + 32 : 48;
-            const int i1 = pmod(cy + t1 / 7 - 3, nRy) * nRx + pmod(cx + t1 % 7 - 3, nRx);
-            v[wl][lane] = rp[i0];
-            if (two) v[wl][lane + 32] = rp[i1];
-            __syncwarp();
-            float a0 = 0.0f, a1 = 0.0f;
-#pragma unroll
-            for (int j = 0; j < 49; ++j) {
-                const float vj = v[wl][j];
-                a0 = fmaf(m0[j], vj, a0);
-                a1 = fmaf(m1[j], vj, a1);
+        const int hi = level_off[lev + 1];
+        int ib = level_off[lev] + wl;
+        ana::BlockIn cur, nxt;
+        int2 c1 = make_int2(0, 0);
+        if (ib < hi) {
+            cur.place(cells[ib], nRx, nRy);
+            cur.fetch(rp);
+            c1 = cells[min(ib + nw, hi - 1)];
+        }
+        for (; ib < hi; ib += nw) {
+            nxt.place(c1, nRx, nRy);
+            if (ib + nw < hi) {
+                nxt.fetch(rp);
+                c1 = cells[min(ib + 2 * nw, hi - 1)];
             }
-            __syncwarp();
-            rp[i0] = a0;
-            if (two) rp[i1] = a1;
+            float a0, a1;
+            ana::block_product(M, cur, v[wl], a0, a1);
+            rp[cur.i0] = a0;
+            if (lane + 32 < 49) rp[cur.i1] = a1;
+            cur = nxt;
         }
         __syncthreads();     // the next level reads what this one wrote
     }
@@ -433,15 +431,24 @@ cudaError_t launch_block_seq(float* r, int NR, int ne, const float* M49, const i
                              int nRy, cudaStream_t st)
 {
     if (nobs <= 0) return cudaSuccess;
-    block_seq_kernel<<<ne, 64, 0, st>>>(r, NR, M49, obs_block0, nobs, nRx, nRy);
+    block_seq_kernel<<<ne, 32, 0, st>>>(r, NR, M49, obs_block0, nobs, nRx, nRy);
     return cudaGetLastError();
 }
 
-cudaError_t launch_block_levels(float* r, int NR, int ne, const float* M49, const int* obs_block0, const int* order,
-                                const int* level_off, int nlev, int nRx, int nRy, cudaStream_t st)
+cudaError_t launch_block_levels(float* r, int NR, int ne, const float* M49, const int* obs_block0, int nobs,
+                                const int* cells, const int* level_off, int nlev, int nRx, int nRy, cudaStream_t st)
 {
     if (nlev <= 0 || ne <= 0) return cudaSuccess;
-    block_levels_kernel<<<ne, BL_THREADS, 0, st>>>(r, NR, M49, obs_block0, order, level_off, nlev, nRx, nRy);
+    // a lattice that closes on itself chains its blocks (1521 levels of one): a
+    // warp along the chain where each has an SM to itself (100 particles: 4.9 ms
+    // per analysis, 5.4 by levels; 1000: 13.7 and 13.0), else the levels
+    if (nobs < 2 * nlev && ne <= tc::sm_count())
+        return launch_block_seq(r, NR, ne, M49, obs_block0, nobs, nRx, nRy, st);
+    // 16 warps (of 128 registers a thread) are resident per SM
+    int warps = 2;
+    while (warps < BL_WARPS && (long long)ne * warps * 2 <= 16LL * tc::sm_count()) warps *= 2;
+    block_levels_kernel<<<ne, 32 * warps, 0, st>>>(r, NR, M49, reinterpret_cast<const int2*>(cells), level_off, nlev,
+                                                   nRx, nRy);
     return cudaGetLastError();
 }
 

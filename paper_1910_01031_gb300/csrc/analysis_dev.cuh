@@ -1093,32 +1093,134 @@ __device__ __forceinline__ void form_r_block(uint64_t seed, uint32_t t, uint32_t
     }
 }
 
-// CTA of at least 64 threads: the 7x7 block roots of every observation of
-// particle p applied in observation order (eq. Psquareroot, Sec. 4.6)
-__device__ __forceinline__ void block_seq_cta(float* __restrict__ r, int NR, const float* __restrict__ M49,
-                                              const int* __restrict__ block0, int nobs, int nRx, int nRy, int p)
-{
-    __shared__ float v[49];
-    __shared__ int idx[49];
-    float* rp = r + (long long)p * NR;
-    const int t = threadIdx.x;
-    for (int l = 0; l < nobs; ++l) {
-        __syncthreads();
-        if (t < 49) {
-            const int dxo = t % 7 - 3, dyo = t / 7 - 3;
-            const int a = pmod(block0[2 * l] + dxo, nRx), b = pmod(block0[2 * l + 1] + dyo, nRy);
-            idx[t] = b * nRx + a;
-            v[t] = rp[idx[t]];
-        }
-        __syncthreads();
-        if (t < 49) {
-            float acc = 0.0f;
-#pragma unroll 7
-            for (int j = 0; j < 49; ++j) acc = fmaf(M49[t * 49 + j], v[j], acc);
-            rp[idx[t]] = acc;
+// Local blocks r_l <- M49 r_l (7 x 7 coarse points around an observation), a
+// warp per block: lane t computes outputs t and t + 32 (< 49), its two rows
+// of M49 in registers, the 49 inputs read from shared memory four at a time.
+// A block costs the round trip of its inputs to L2 and 49 dependent products;
+// the inputs of the next block are loaded during the products where the two
+// share no point.
+struct BlockRoot {
+    float m0[49], m1[49];
+    __device__ __forceinline__ void load(const float* __restrict__ M49)
+    {
+        const int lane = threadIdx.x & 31;
+#pragma unroll
+        for (int j = 0; j < 49; ++j) {
+            m0[j] = __ldg(M49 + lane * 49 + j);
+            m1[j] = lane + 32 < 49 ? __ldg(M49 + (lane + 32) * 49 + j) : 0.0f;
         }
     }
-    __syncthreads();
+};
+struct BlockIn {
+    int i0, i1;      // this lane's points
+    float x0, x1;    // and their values
+    __device__ __forceinline__ void place(int2 c, int nRx, int nRy)
+    {
+        const int lane = threadIdx.x & 31, t1 = lane + 32 < 49 ? lane + 32 : 48;
+        auto wrap = [](int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); };
+        i0 = wrap(c.y + lane / 7 - 3, nRy) * nRx + wrap(c.x + lane % 7 - 3, nRx);
+        i1 = wrap(c.y + t1 / 7 - 3, nRy) * nRx + wrap(c.x + t1 % 7 - 3, nRx);
+    }
+    __device__ __forceinline__ void fetch(const float* rp)
+    {
+        // in place: the compiler would sink the loads towards their use
+        asm volatile("ld.global.f32 %0, [%1];" : "=f"(x0) : "l"(rp + i0) : "memory");
+        asm volatile("ld.global.f32 %0, [%1];" : "=f"(x1) : "l"(rp + i1) : "memory");
+    }
+};
+// v: 52 floats of shared memory, 16-byte aligned, owned by the warp
+__device__ __forceinline__ void block_product(const BlockRoot& M, const BlockIn& B, float* v, float& a0, float& a1)
+{
+    const int lane = threadIdx.x & 31;
+    v[lane] = B.x0;
+    if (lane + 32 < 49) v[lane + 32] = B.x1;
+    __syncwarp();
+    a0 = a1 = 0.0f;
+#pragma unroll
+    for (int q = 0; q < 13; ++q) {
+        const float4 w = *reinterpret_cast<const float4*>(v + 4 * q);
+        const float c[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (4 * q + u < 49) {
+                a0 = fmaf(M.m0[4 * q + u], c[u], a0);
+                a1 = fmaf(M.m1[4 * q + u], c[u], a1);
+            }
+    }
+    __syncwarp();
+}
+
+// warp: the blocks of particle p in observation order.  Blocks that follow
+// each other mostly share points, so a block's inputs are loaded two blocks
+// ahead and those of the two blocks before it, then written, come from their
+// outputs in shared memory (v: 3 x 52 floats, 16-byte aligned): a block costs
+// its products, not the round trip through L2 of its predecessor's outputs.
+__device__ __forceinline__ void block_seq_warp(float* r, int NR, const float* __restrict__ M49,
+                                               const int* __restrict__ block0, int nobs, int nRx, int nRy, int p,
+                                               float* v)
+{
+    if (nobs <= 0) return;
+    const int lane = threadIdx.x & 31, t1 = lane + 32 < 49 ? lane + 32 : 48;
+    float* rp = r + (long long)p * NR;
+    const int2* cells = reinterpret_cast<const int2*>(block0);
+    BlockRoot M;
+    M.load(M49);
+    const int lx0 = lane % 7, ly0 = lane / 7, lx1 = t1 % 7, ly1 = t1 / 7;
+    // the block's place relative to another's, in (-n / 2, n / 2]
+    auto offset = [](int a, int b, int n) {
+        const int d = a - b;
+        return 2 * d > n ? d - n : (2 * d <= -n ? d + n : d);
+    };
+    int2 cm = cells[0], c0 = cm, c1 = cells[min(1, nobs - 1)], c2 = cells[min(2, nobs - 1)];
+    // blocks ahead whose inputs are brought to L2 (DRAM takes longer than two blocks)
+    constexpr int SEQ_AHEAD = 8;
+    int2 ca = cells[min(SEQ_AHEAD, nobs - 1)];
+    BlockIn cur, nxt;
+    cur.place(c0, nRx, nRy);
+    cur.fetch(rp);
+    nxt.place(c1, nRx, nRy);
+    nxt.fetch(rp);
+    float* const out0 = v + 52;
+#pragma unroll 4
+    for (int l = 0; l < nobs; ++l) {
+        const int2 c3 = cells[min(l + 3, nobs - 1)];
+        if (l + SEQ_AHEAD < nobs) {
+            BlockIn q;
+            q.place(ca, nRx, nRy);
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(rp + q.i0));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(rp + q.i1));
+            ca = cells[min(l + 1 + SEQ_AHEAD, nobs - 1)];
+        }
+        BlockIn far;
+        far.place(c2, nRx, nRy);
+        far.fetch(rp);
+        float a0, a1;
+        block_product(M, cur, v, a0, a1);
+        const int cur0 = 52 * (l & 1);
+        rp[cur.i0] = a0;
+        out0[cur0 + lane] = a0;
+        if (lane + 32 < 49) {
+            rp[cur.i1] = a1;
+            out0[cur0 + lane + 32] = a1;
+        }
+        __syncwarp();
+        // the next block's inputs were loaded before this block and the one before wrote
+        const int dx = offset(c1.x, c0.x, nRx), dy = offset(c1.y, c0.y, nRy);
+        const int ex = offset(c1.x, cm.x, nRx), ey = offset(c1.y, cm.y, nRy);
+        auto latest = [&](int t, int lx, int ly, float g) {
+            const bool in0 = ((unsigned)(lx + dx) < 7u) & ((unsigned)(ly + dy) < 7u);
+            const bool inm = ((unsigned)(lx + ex) < 7u) & ((unsigned)(ly + ey) < 7u) & (l > 0);
+            const int k = in0 ? cur0 + 7 * dy + dx + t : (inm ? (52 - cur0) + 7 * ey + ex + t : 0);
+            const float w = out0[k];
+            return in0 | inm ? w : g;
+        };
+        cur.i0 = nxt.i0;
+        cur.i1 = nxt.i1;
+        cur.x0 = latest(lane, lx0, ly0, nxt.x0);
+        cur.x1 = latest(t1, lx1, ly1, nxt.x1);
+        nxt = far;
+        cm = c0; c0 = c1; c1 = c2; c2 = c3;
+    }
 }
 
 }  // namespace ana

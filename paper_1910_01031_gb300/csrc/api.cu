@@ -967,8 +967,13 @@ int iewpf_create(const iewpf_params_t* params, const double* mooring_xy, iewpf_c
         std::vector<int> level_off;
         block_levels(b0.data(), nobs, ctx->C.nRx, ctx->C.nRy, order, level_off);
         ctx->nblev = (int)level_off.size() - 1;
-        if ((rc = dalloc(ctx, &ctx->d_border, nobs)) || (rc = dalloc(ctx, &ctx->d_blevel, level_off.size())) ||
-            cudaMemcpy(ctx->d_border, order.data(), sizeof(int) * nobs, cudaMemcpyHostToDevice) != cudaSuccess ||
+        std::vector<int> places(2 * (size_t)nobs);
+        for (int i = 0; i < nobs; ++i) {
+            places[2 * i] = b0[2 * order[i]];
+            places[2 * i + 1] = b0[2 * order[i] + 1];
+        }
+        if ((rc = dalloc(ctx, &ctx->d_border, 2 * (size_t)nobs)) || (rc = dalloc(ctx, &ctx->d_blevel, level_off.size())) ||
+            cudaMemcpy(ctx->d_border, places.data(), sizeof(int) * 2 * nobs, cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemcpy(ctx->d_blevel, level_off.data(), sizeof(int) * level_off.size(), cudaMemcpyHostToDevice) !=
                 cudaSuccess)
             return bail(rc ? rc : IEWPF_ECUDA);
@@ -1112,8 +1117,8 @@ int iewpf_assimilate(iewpf_ctx_t* ctx, const iewpf_obs_t* obs, iewpf_diag_t* dia
     KL(1, launch_form_r(ctx->P.seed, ctx->cycle, sb + 1, sb + 2, (int)ctx->NR, ne, ctx->d_coef, ctx->d_scal,
                      ctx->d_alpha, ctx->d_r, ctx->st));
     if (mooring && ctx->nblev > 0) {
-        KL(1, launch_block_levels(ctx->d_r, (int)ctx->NR, ne, ctx->d_M49, ctx->d_block0, ctx->d_border, ctx->d_blevel,
-                                  ctx->nblev, ctx->C.nRx, ctx->C.nRy, ctx->st));
+        KL(1, launch_block_levels(ctx->d_r, (int)ctx->NR, ne, ctx->d_M49, ctx->d_block0, nobs, ctx->d_border,
+                                  ctx->d_blevel, ctx->nblev, ctx->C.nRx, ctx->C.nRy, ctx->st));
     } else {
         KL(1, launch_block_seq(ctx->d_r, (int)ctx->NR, ne, ctx->d_M49, ctx->d_block0, nobs, ctx->C.nRx, ctx->C.nRy,
                                ctx->st));

@@ -352,13 +352,14 @@ __global__ void b_form_r(BatchDev B)
     }
 }
 
-__global__ void b_block_seq(BatchDev B)
+__global__ void __launch_bounds__(32) b_block_seq(BatchDev B)
 {
+    __shared__ __align__(16) float v[3 * 52];
     const long long* pre = space(B, SP_PART);
     for (long long q = blockIdx.x; q < pre[B.n]; q += gridDim.x) {
         const int i = find_inst(pre, B.n, q);
         const BInst& I = B.inst[i];
-        ana::block_seq_cta(I.r, (int)I.NR, I.M49, I.block0, I.nobs, I.C.nRx, I.C.nRy, (int)(q - pre[i]));
+        ana::block_seq_warp(I.r, (int)I.NR, I.M49, I.block0, I.nobs, I.C.nRx, I.C.nRy, (int)(q - pre[i]), v);
     }
 }
 
@@ -658,7 +659,7 @@ static cudaError_t capture_analysis(BatchImpl& b, cudaStream_t st)
     b_dots<<<grid_for(b_dots, ana::DOT_THREADS, items(b, SP_DOT)), ana::DOT_THREADS, 0, st>>>(B);
     b_sync<<<b.n, ana::SYNC_THREADS, 0, st>>>(B);
     b_form_r<<<grid_for(b_form_r, 256, (items(b, SP_NRM) + 255) / 256), 256, 0, st>>>(B);
-    b_block_seq<<<grid_for(b_block_seq, 64, items(b, SP_PART)), 64, 0, st>>>(B);
+    b_block_seq<<<grid_for(b_block_seq, 32, items(b, SP_PART)), 32, 0, st>>>(B);
     b_soar<true><<<grid_for(b_soar<true>, 256, (items(b, SP_FR) + 255) / 256), 256, 0, st>>>(B);
     if ((e = launch_fine<true>(b, st)) != cudaSuccess) return e;
     b_count<<<(b.n + 127) / 128, 128, 0, st>>>(B, 1);

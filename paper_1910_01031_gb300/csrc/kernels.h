@@ -204,12 +204,13 @@ cudaError_t launch_form_r(uint64_t seed, uint32_t t, uint32_t s_xi, uint32_t s_n
                           cudaStream_t st);
 cudaError_t launch_block_seq(float* r, int NR, int ne, const float* M49, const int* obs_block0, int nobs, int nRx,
                              int nRy, cudaStream_t st);
-// the same products level by level (block_levels: order and level_off in
-// device memory, nlev levels; the blocks of a level pairwise share no coarse
-// point), one CTA per particle whose warps share each level's blocks, the
-// same arithmetic as block_seq, so the result is block_seq's bit for bit
-cudaError_t launch_block_levels(float* r, int NR, int ne, const float* M49, const int* obs_block0, const int* order,
-                                const int* level_off, int nlev, int nRx, int nRy, cudaStream_t st);
+// the same products level by level (cells: the blocks' places in the order of
+// block_levels, level_off its offsets, both in device memory; nlev levels; the
+// blocks of a level pairwise share no coarse point), one CTA per particle
+// whose warps share each level's blocks, or block_seq itself where the levels
+// are a chain; the same arithmetic, so the result is block_seq's bit for bit
+cudaError_t launch_block_levels(float* r, int NR, int ne, const float* M49, const int* obs_block0, int nobs,
+                                const int* cells, const int* level_off, int nlev, int nRx, int nRy, cudaStream_t st);
 // host: level of each block (0 when it shares no coarse point with an earlier
 // block, else one more than the highest level among the earlier blocks it
 // overlaps; blocks are 7 x 7 coarse points around block0 on the periodic

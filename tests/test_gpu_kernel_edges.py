@@ -155,3 +155,22 @@ def test_grouped_sweeps_equal_a_warp_per_particle(m, spacing, ne):
     d = single.assimilate(None, y)
     assert diag[0, 0] == d["w_target"] and diag[0, 1] == d["beta"] and diag[0, 2] == 0
     assert np.array_equal(batch.instances[0].get_state(), single.get_state())
+
+
+@pytest.mark.parametrize("positions", ["same", "overlapping", "wrapping", "apart"])
+@pytest.mark.parametrize("n", [1, 2, 3, 13])
+def test_local_blocks_in_sequence(n, positions):
+    """Local blocks applied one after another (inputs loaded two blocks ahead, the two blocks before patched
+    in): fewer blocks than the look-ahead, blocks on one place, sharing points with one or both predecessors,
+    over the periodic edges and apart, against the oracle's products in FP64 at 1e-5 of the state."""
+    cfg = synth.Config("edge", 96, 93, n_particles=3, n_obs=n)
+    ens, P = ensemble(cfg), oracle_problem(cfg)
+    U32, U64 = start_state(cfg, 3)
+    ens.set_state(U32)
+    step = {"same": (0, 0), "overlapping": (7, 4), "wrapping": (40, 88), "apart": (29, 24)}[positions]
+    cells = np.array([[(5 + step[0] * k) % 96, (3 + step[1] * k) % 93] for k in range(n)])
+    xy = synth.cell_positions(cfg, cells)
+    y = synth.obs_from_state(cfg, synth.initial_particle(cfg, 77, seed=5), cells, synth.obs_noise(cfg, n, 0))
+    ens.assimilate(xy, y)
+    ref, _ = O.assimilate(P, U64, [tuple(c) for c in cells], y, t=0)
+    assert rel_l2(ens.get_state(), ref) <= 1e-5
