@@ -11,6 +11,8 @@ namespace iewpf {
 
 namespace {
 
+// dynamic shared memory of cholesky_small_kernel (n <= 159) at most
+constexpr int kCholSmem = 212 * 1024;
 // dynamic shared memory of a CTA of the grouped sweeps at most
 constexpr int kSolveGroupSmem = 224 * 1024;
 
@@ -48,24 +50,26 @@ cholesky_kernel(double* __restrict__ A, int n, int* __restrict__ colptr, int* ro
                 int* nzlist, double* __restrict__ rdiag, int* plan)
 {
     ana::cholesky_cta(A, n, colptr, rowidx, flag, nzlist);
-    ana::solve_plan_cta(A, n, colptr, rowidx, rdiag, plan);
+    ana::solve_plan_cta<false>(A, n, n, colptr, rowidx, rdiag, plan);
 }
 
-// the same factorisation on a copy in shared memory (n * n doubles + n ints)
+// the same factorisation on a copy in shared memory (n rows of an odd
+// number of doubles, then chol_levels_ints(n) >= n ints)
 __global__ void __launch_bounds__(1024)
 cholesky_small_kernel(double* __restrict__ A, int n, int* __restrict__ colptr, int* __restrict__ rowidx,
                       int* __restrict__ flag, double* __restrict__ rdiag, int* plan)
 {
     extern __shared__ double sA[];
-    int* work = reinterpret_cast<int*>(sA + (long long)n * n);
+    const int ld = n | 1;
+    int* work = reinterpret_cast<int*>(sA + n * ld);
     __shared__ int bad;
     if (threadIdx.x == 0) bad = 0;
-    for (int q = threadIdx.x; q < n * n; q += blockDim.x) sA[q] = A[q];
+    for (int q = threadIdx.x; q < n * n; q += blockDim.x) sA[q / n * ld + q % n] = A[q];
     __syncthreads();
-    ana::cholesky_factor_cta(sA, n, work, &bad);
-    for (int q = threadIdx.x; q < n * n; q += blockDim.x) A[q] = sA[q];
-    ana::csc_cta(sA, n, colptr, rowidx);
-    ana::solve_plan_cta(sA, n, colptr, rowidx, rdiag, plan);
+    if (!ana::cholesky_levels_cta(sA, n, ld, work, &bad)) ana::cholesky_factor_cta(sA, n, ld, work, &bad);
+    for (int q = threadIdx.x; q < n * n; q += blockDim.x) A[q] = sA[q / n * ld + q % n];
+    ana::csc_cta(sA, n, ld, colptr, rowidx);
+    ana::solve_plan_cta<true>(sA, n, ld, colptr, rowidx, rdiag, plan);
     if (threadIdx.x == 0 && bad) atomicOr(flag, FLAG_NOTPD);
 }
 
@@ -305,10 +309,10 @@ cudaError_t launch_cholesky(double* M, int n, int* colptr, int* rowidx, int* fla
     // small systems (drifter layouts change every cycle) factor in shared memory
     const size_t smem = (size_t)n * n * sizeof(double) + (size_t)n * sizeof(int);
     if (n >= 1 && smem <= 200 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(cholesky_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
+        cudaError_t e = tc::smem_attr_once<cholesky_small_kernel>(kCholSmem);
         if (e != cudaSuccess) return e;
-        cholesky_small_kernel<<<1, 1024, smem, st>>>(M, n, colptr, rowidx, flag, rdiag, plan);
+        const size_t bytes = (size_t)n * (n | 1) * sizeof(double) + ana::chol_levels_ints(n) * sizeof(int);
+        cholesky_small_kernel<<<1, 1024, bytes, st>>>(M, n, colptr, rowidx, flag, rdiag, plan);
         return cudaGetLastError();
     }
     // rowidx doubles as the per-column work list during the factorisation

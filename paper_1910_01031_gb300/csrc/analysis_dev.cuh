@@ -121,24 +121,26 @@ __device__ __forceinline__ void hqht_one(const double* __restrict__ K, int R, co
 // CTA; the update of column k touches only rows with a non-zero in it, so
 // block-diagonal and banded matrices cost their fill, not n^3/3.  A may live
 // in global or shared memory; nzlist holds n ints.  The strict upper triangle
-// is zeroed; *bad (shared) is set for a non-positive pivot.
-__device__ __forceinline__ void cholesky_factor_cta(double* __restrict__ A, int n, int* __restrict__ nzlist, int* bad)
+// is zeroed; *bad (shared) is set for a non-positive pivot.  ld: doubles from
+// row to row (odd in shared memory, where columns are read too).
+__device__ __forceinline__ void cholesky_factor_cta(double* __restrict__ A, int n, int ld, int* __restrict__ nzlist,
+                                                    int* bad)
 {
     __shared__ int nnz;
     __shared__ double piv;
     for (int k = 0; k < n; ++k) {
         if (threadIdx.x == 0) {
-            const double dkk = A[(long long)k * n + k];
+            const double dkk = A[(long long)k * ld + k];
             if (!(dkk > 0.0)) *bad = 1;
             piv = dkk > 0.0 ? sqrt(dkk) : 1.0;
-            A[(long long)k * n + k] = piv;
+            A[(long long)k * ld + k] = piv;
             nnz = 0;
         }
         __syncthreads();
         for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) {
-            const double v = A[(long long)i * n + k];
+            const double v = A[(long long)i * ld + k];
             if (v != 0.0) {
-                A[(long long)i * n + k] = v / piv;
+                A[(long long)i * ld + k] = v / piv;
                 nzlist[atomicAdd(&nnz, 1)] = i;
             }
         }
@@ -147,43 +149,191 @@ __device__ __forceinline__ void cholesky_factor_cta(double* __restrict__ A, int 
         const long long pairs = (long long)m * m;
         for (long long q = threadIdx.x; q < pairs; q += blockDim.x) {
             const int i = nzlist[q / m], j = nzlist[q % m];
-            if (j <= i) A[(long long)i * n + j] = fma(-A[(long long)i * n + k], A[(long long)j * n + k], A[(long long)i * n + j]);
+            if (j <= i) A[(long long)i * ld + j] = fma(-A[(long long)i * ld + k], A[(long long)j * ld + k], A[(long long)i * ld + j]);
         }
         __syncthreads();
     }
     for (long long q = threadIdx.x; q < (long long)n * n; q += blockDim.x) {
         const int i = (int)(q / n), j = (int)(q % n);
-        if (j > i) A[q] = 0.0;
+        if (j > i) A[(long long)i * ld + j] = 0.0;
     }
     __syncthreads();
+}
+
+// CTA: counts p[1..n] to offsets p[0..n] in place, by warp 0
+__device__ __forceinline__ void prefix_cta(int* p, int n)
+{
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        int base = 0;
+        for (int t0 = 1; t0 <= n; t0 += 32) {
+            const int t = t0 + lane;
+            int v = t <= n ? p[t] : 0;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int w = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += w;
+            }
+            if (t <= n) p[t] = base + v;
+            base += __shfl_sync(0xffffffffu, v, 31);
+        }
+        if (lane == 0) p[0] = 0;
+    }
+    __syncthreads();
+}
+
+// CTA: rows in increasing index within each level (deterministic), ptr the
+// level boundaries, *nlev their number: every row counts those before it
+__device__ __forceinline__ void level_sort_cta(const int* __restrict__ lev, int n, int* __restrict__ order,
+                                               int* __restrict__ ptr, int* __restrict__ nlev)
+{
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const int li = lev[i];
+        int below = 0, same = 0, top = 0;
+        for (int j = 0; j < n; ++j) {
+            const int lj = lev[j];
+            below += lj < li;
+            same += lj == li && j < i;
+            top = max(top, lj);
+        }
+        order[below + same] = i;
+        if (same == 0) ptr[li] = below;
+        if (i == 0) {
+            ptr[top + 1] = n;
+            *nlev = top + 1;
+        }
+    }
+}
+
+// The factorisation of cholesky_factor_cta level by level, A in shared memory:
+// a column depends on those that its row has entries in, so the columns of one
+// level of the elimination tree are factored together.  FP64 latency bounds a
+// column (a square root, then a division: about 3500 cycles), so what counts
+// is how many follow one another: 128 for 64 drifters column by column, a few
+// by levels where most of them do not interact (factor and plan 258 us, now
+// 69).  Left-looking, with every entry's products in the order of
+// cholesky_factor_cta and its rules for zeros: the same bits.  False, with A
+// unchanged, when the levels are more than a quarter of the columns (a thread
+// per entry would then have too many products) or the columns few.
+// n <= 1024; work:
+// chol_levels_ints(n) ints of shared memory.
+__host__ __device__ __forceinline__ int chol_levels_ints(int n) { return 2 * n * ((n + 31) / 32) + 4 * n + 3; }
+__device__ __forceinline__ bool cholesky_levels_cta(double* A, int n, int ld, int* work, int* bad)
+{
+    if (n < 32) return false;
+    const int nw = (n + 31) / 32, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    unsigned* const col = reinterpret_cast<unsigned*>(work);   // [n][nw] rows below the diagonal of each column
+    unsigned* const row = col + n * nw;                        // [n][nw] columns before the diagonal of each row
+    int* const lev = work + 2 * n * nw;
+    int* const order = lev + n;
+    int* const first = order + n;                              // [n + 1]
+    int* const ptr = first + n + 1;                            // [n + 1], then the number of levels
+    for (int k = warp; k < n; k += warps) {
+        for (int w = 0; w < nw; ++w) {
+            const int i = 32 * w + lane;
+            const unsigned b = __ballot_sync(0xffffffffu, i > k && i < n && A[i * ld + k] != 0.0);
+            if (lane == 0) col[k * nw + w] = b;
+        }
+        if (lane == 0) lev[k] = 0;
+    }
+    __syncthreads();
+    // fill: a column's first row below the diagonal is its parent, which
+    // inherits its other rows
+    if (warp == 0)
+        for (int k = 0; k < n; ++k) {
+            const unsigned mine = lane < nw ? col[k * nw + lane] : 0u;
+            const unsigned any = __ballot_sync(0xffffffffu, mine != 0u);
+            if (any == 0u) continue;
+            const int w0 = __ffs(any) - 1;
+            const int bit = __ffs(__shfl_sync(0xffffffffu, mine, w0)) - 1, p = 32 * w0 + bit;
+            if (lane < nw) col[p * nw + lane] |= lane == w0 ? mine & ~(1u << bit) : mine;
+            if (lane == 0) lev[p] = max(lev[p], lev[k] + 1);
+            __syncwarp();
+        }
+    __syncthreads();
+    for (int j = warp; j < n; j += warps)
+        for (int w = 0; w < nw; ++w) {
+            const int k = 32 * w + lane;
+            const unsigned b = __ballot_sync(0xffffffffu, k < j && ((col[min(k, n - 1) * nw + (j >> 5)] >> (j & 31)) & 1u));
+            if (lane == 0) row[j * nw + w] = b;
+        }
+    level_sort_cta(lev, n, order, ptr, ptr + n + 1);
+    __syncthreads();
+    const int nlev = ptr[n + 1];
+    if (4 * nlev > n) return false;
+    // first[t]: entries below the diagonal of the columns before position t
+    for (int t = threadIdx.x; t < n; t += blockDim.x) {
+        int c = 0;
+        for (int w = 0; w < nw; ++w) c += __popc(col[order[t] * nw + w]);
+        first[t + 1] = c;
+    }
+    __syncthreads();
+    prefix_cta(first, n);
+    // entry (i, j) less its products over the columns of row j, in their order
+    auto reduced = [&](int i, int j) {
+        double acc = A[i * ld + j];
+        for (int w = 0; w <= j >> 5; ++w)
+            for (unsigned b = row[j * nw + w]; b; b &= b - 1u) {
+                const int k = 32 * w + __ffs(b) - 1;
+                const double ajk = A[j * ld + k], aik = A[i * ld + k];
+                if (ajk != 0.0 && aik != 0.0) acc = fma(-aik, ajk, acc);
+            }
+        return acc;
+    };
+    for (int l = 0; l < nlev; ++l) {
+        // a thread per pivot, then a thread per entry
+        for (int t = ptr[l] + threadIdx.x; t < ptr[l + 1]; t += blockDim.x) {
+            const int j = order[t];
+            const double d = reduced(j, j);
+            if (!(d > 0.0)) *bad = 1;
+            A[j * ld + j] = d > 0.0 ? sqrt(d) : 1.0;
+        }
+        __syncthreads();
+        for (int q = first[ptr[l]] + threadIdx.x; q < first[ptr[l + 1]]; q += blockDim.x) {
+            int lo = ptr[l], hi = ptr[l + 1];           // first[lo] <= q < first[hi]
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (first[mid] <= q) lo = mid;
+                else hi = mid;
+            }
+            const int j = order[lo];
+            int rank = q - first[lo], w = 0, c;
+            while (rank >= (c = __popc(col[j * nw + w]))) rank -= c, ++w;
+            unsigned b = col[j * nw + w];
+            for (; rank > 0; --rank) b &= b - 1u;
+            const int i = 32 * w + __ffs(b) - 1;
+            const double v = reduced(i, j);
+            A[i * ld + j] = v != 0.0 ? v / A[j * ld + j] : v;
+        }
+        __syncthreads();
+    }
+    for (int i = warp; i < n; i += warps)
+        for (int k = i + 1 + lane; k < n; k += 32) A[i * ld + k] = 0.0;
+    __syncthreads();
+    return true;
 }
 
 // The factor's columns as CSC of the strictly lower part, rows increasing:
 // one warp per column counts (ballots), a prefix sum gives colptr, and the
 // warps write the row lists in order.
-__device__ __forceinline__ void csc_cta(const double* __restrict__ L, int n, int* __restrict__ colptr,
-                                        int* __restrict__ rowidx)
+__device__ __forceinline__ void csc_cta(const double* __restrict__ L, int n, int ld, int* colptr, int* __restrict__ rowidx)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int k = warp; k < n; k += nw) {
         int cnt = 0;
         for (int i0 = k + 1; i0 < n; i0 += 32) {
             const int i = i0 + lane;
-            cnt += __popc(__ballot_sync(0xffffffffu, i < n && L[(long long)i * n + k] != 0.0));
+            cnt += __popc(__ballot_sync(0xffffffffu, i < n && L[(long long)i * ld + k] != 0.0));
         }
         if (lane == 0) colptr[k + 1] = cnt;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        colptr[0] = 0;
-        for (int k = 0; k < n; ++k) colptr[k + 1] += colptr[k];
-    }
-    __syncthreads();
+    prefix_cta(colptr, n);
     for (int k = warp; k < n; k += nw) {
         int pos = colptr[k];
         for (int i0 = k + 1; i0 < n; i0 += 32) {
             const int i = i0 + lane;
-            const bool nz = i < n && L[(long long)i * n + k] != 0.0;
+            const bool nz = i < n && L[(long long)i * ld + k] != 0.0;
             const unsigned bal = __ballot_sync(0xffffffffu, nz);
             if (nz) rowidx[pos + __popc(bal & ((1u << lane) - 1u))] = i;
             pos += __popc(bal);
@@ -203,8 +353,8 @@ __device__ __forceinline__ void cholesky_cta(double* __restrict__ A, int n, int*
     __syncthreads();
     if (threadIdx.x == 0) bad = 0;
     __syncthreads();
-    cholesky_factor_cta(A, n, nzlist, &bad);
-    csc_cta(A, n, colptr, rowidx);
+    cholesky_factor_cta(A, n, n, nzlist, &bad);
+    csc_cta(A, n, n, colptr, rowidx);
     if (threadIdx.x == 0 && bad) atomicOr(flag, FLAG_NOTPD);
 }
 
@@ -237,80 +387,104 @@ __host__ __device__ inline SolvePlan solve_plan_view(int* base, int n)
     return P;
 }
 
-// rows in increasing index within each level (deterministic); ptr gets the
-// level boundaries; one thread
-__device__ __forceinline__ int level_sort(const int* __restrict__ lev, int n, int* __restrict__ order,
-                                          int* __restrict__ ptr)
+// CTA: lev[i] = 1 + the largest level among the j with entry(i, j), by rounds
+// over all i until none grows (levels only grow, so a round may read those
+// that it is raising); lev in shared memory
+template <class F>
+__device__ __forceinline__ void levels_smem_cta(int* lev_, int n, F entry)
 {
-    int nl = 0;
-    for (int i = 0; i < n; ++i) nl = max(nl, lev[i] + 1);
-    for (int l = 0; l <= nl; ++l) ptr[l] = 0;
-    for (int i = 0; i < n; ++i) ptr[lev[i] + 1]++;
-    for (int l = 0; l < nl; ++l) ptr[l + 1] += ptr[l];
-    for (int i = 0; i < n; ++i) order[ptr[lev[i]]++] = i;
-    for (int l = nl; l > 0; --l) ptr[l] = ptr[l - 1];
-    ptr[0] = 0;
-    return nl;
+    volatile int* lev = lev_;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) lev[i] = 0;
+    __syncthreads();
+    bool grew = true;
+    while (grew) {
+        grew = false;
+        for (int i = warp; i < n; i += nw) {
+            int m = -1;
+            for (int j0 = 0; j0 < n; j0 += 32) {
+                const int j = j0 + lane;
+                if (j < n && entry(i, j)) m = max(m, lev[j]);
+            }
+            m = __reduce_max_sync(0xffffffffu, m) + 1;
+            if (m > lev[i]) {
+                grew = true;
+                __syncwarp();
+                if (lane == 0) lev[i] = m;
+            }
+            __syncwarp();
+        }
+        grew = __syncthreads_or(grew);
+    }
 }
 
 // CTA: reciprocal diagonal, CSR of L below the diagonal and both level
-// schedules; after csc_cta (colptr/rowidx complete)
-__device__ __forceinline__ void solve_plan_cta(const double* __restrict__ L, int n, const int* __restrict__ colptr,
+// schedules; after csc_cta (colptr/rowidx complete).  The levels are kept in
+// shared memory where they fit, and with L itself there (SMEM) the rows'
+// non-zeros are read from it (64 drifters: one thread or warp going row by
+// row through global memory took about 90 us, rounds over all rows 10).
+constexpr int PLAN_LEV = 2048;
+template <bool SMEM>
+__device__ __forceinline__ void solve_plan_cta(const double* __restrict__ L, int n, int ld, const int* __restrict__ colptr,
                                                const int* __restrict__ rowidx, double* __restrict__ rdiag,
                                                int* plan_base)
 {
     const SolvePlan P = solve_plan_view(plan_base, n);
+    __shared__ int slev[PLAN_LEV];
+    int* const lev = n <= PLAN_LEV ? slev : P.lev;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) rdiag[i] = 1.0 / L[(long long)i * n + i];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) rdiag[i] = 1.0 / L[(long long)i * ld + i];
     for (int i = warp; i < n; i += nw) {
         int cnt = 0;
         for (int j0 = 0; j0 < i; j0 += 32) {
             const int j = j0 + lane;
-            cnt += __popc(__ballot_sync(0xffffffffu, j < i && L[(long long)i * n + j] != 0.0));
+            cnt += __popc(__ballot_sync(0xffffffffu, j < i && L[(long long)i * ld + j] != 0.0));
         }
         if (lane == 0) P.rowptr[i + 1] = cnt;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        P.rowptr[0] = 0;
-        for (int i = 0; i < n; ++i) P.rowptr[i + 1] += P.rowptr[i];
-    }
-    __syncthreads();
+    prefix_cta(P.rowptr, n);
     for (int i = warp; i < n; i += nw) {
         int pos = P.rowptr[i];
         for (int j0 = 0; j0 < i; j0 += 32) {
             const int j = j0 + lane;
-            const bool nz = j < i && L[(long long)i * n + j] != 0.0;
+            const bool nz = j < i && L[(long long)i * ld + j] != 0.0;
             const unsigned bal = __ballot_sync(0xffffffffu, nz);
             if (nz) P.colidx[pos + __popc(bal & ((1u << lane) - 1u))] = j;
             pos += __popc(bal);
         }
     }
     __syncthreads();
-    // forward levels: 1 + the largest level among the row's columns
-    if (warp == 0) {
+    // forward levels: 1 + the largest level among the row's columns.  In shared
+    // memory a warp per row, all rows until nothing changes (as many rounds as
+    // levels); else row after row
+    if (SMEM) {
+        levels_smem_cta(lev, n, [&](int i, int j) { return j < i && L[(long long)i * ld + j] != 0.0; });
+    } else if (warp == 0)
         for (int i = 0; i < n; ++i) {
             int m = -1;
-            for (int q = P.rowptr[i] + lane; q < P.rowptr[i + 1]; q += 32) m = max(m, P.lev[P.colidx[q]]);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-            if (lane == 0) P.lev[i] = m + 1;
+            for (int q = P.rowptr[i] + lane; q < P.rowptr[i + 1]; q += 32) m = max(m, lev[P.colidx[q]]);
+            m = __reduce_max_sync(0xffffffffu, m);
+            if (lane == 0) lev[i] = m + 1;
             __syncwarp();
         }
-        if (lane == 0) P.nlev[0] = level_sort(P.lev, n, P.forder, P.fptr);
-        __syncwarp();
-        // backward levels: 1 + the largest level among the column's rows
+    __syncthreads();
+    level_sort_cta(lev, n, P.forder, P.fptr, P.nlev);
+    __syncthreads();
+    // backward levels: 1 + the largest level among the column's rows
+    if (SMEM) {
+        levels_smem_cta(lev, n, [&](int i, int k) { return k > i && L[(long long)k * ld + i] != 0.0; });
+    } else if (warp == 0)
         for (int i = n - 1; i >= 0; --i) {
             int m = -1;
-            for (int q = colptr[i] + lane; q < colptr[i + 1]; q += 32) m = max(m, P.lev[rowidx[q]]);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-            if (lane == 0) P.lev[i] = m + 1;
+            for (int q = colptr[i] + lane; q < colptr[i + 1]; q += 32) m = max(m, lev[rowidx[q]]);
+            m = __reduce_max_sync(0xffffffffu, m);
+            if (lane == 0) lev[i] = m + 1;
             __syncwarp();
         }
-        if (lane == 0) P.nlev[1] = level_sort(P.lev, n, P.border, P.bptr);
-    }
+    __syncthreads();
+    level_sort_cta(lev, n, P.border, P.bptr, P.nlev + 1);
     __syncthreads();
     for (int t = threadIdx.x; t < n; t += blockDim.x) {
         const int i = P.forder[t], k = P.border[t];

@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(1024) b_cholesky(BatchDev B)
         const BInst& I = B.inst[i];
         if (I.moving_obs) {
             ana::cholesky_cta(I.L, 2 * I.nobs, I.colptr, I.rowidx, I.flag, I.rowidx);
-            ana::solve_plan_cta(I.L, 2 * I.nobs, I.colptr, I.rowidx, I.rdiag, I.plan);
+            ana::solve_plan_cta<false>(I.L, 2 * I.nobs, 2 * I.nobs, I.colptr, I.rowidx, I.rdiag, I.plan);
         }
     }
 }

@@ -174,3 +174,25 @@ def test_local_blocks_in_sequence(n, positions):
     ens.assimilate(xy, y)
     ref, _ = O.assimilate(P, U64, [tuple(c) for c in cells], y, t=0)
     assert rel_l2(ens.get_state(), ref) <= 1e-5
+
+
+@pytest.mark.parametrize("n,spread", [(15, 40), (16, 40), (33, 40), (64, 40), (79, 40), (40, 12), (64, 3), (80, 40)])
+def test_factor_by_levels_equals_column_by_column(n, spread):
+    """Drifter layouts whose factor is made level by level (32 to 159 unknowns that mostly do not interact) or
+    column by column (fewer, more, or clustered), against the batch's, which goes column by column, bit for bit."""
+    cfg = synth.Config("edge", 352, 336, n_particles=2, n_obs=n, c_omega=1)
+    rng = np.random.default_rng(n + spread)
+    cells = np.array([[(spread * (k % 8) + rng.integers(0, 9)) % 352, (spread * (k // 8) + rng.integers(0, 9)) % 336]
+                      for k in range(n)])
+    xy = synth.cell_positions(cfg, cells)
+    batch, single = iewpf.Batch([iewpf.params_from_config(cfg)], None), ensemble(cfg)
+    U = synth.initial_state(cfg, 2, seed=7).astype(np.float32)
+    y = synth.obs_from_state(cfg, synth.initial_particle(cfg, 77, seed=5), cells, synth.obs_noise(cfg, n, 0))
+    for e in (single, batch.instances[0]):
+        e.set_state(U)
+    diag = batch.cycle(2, [(xy, y)])
+    single.forecast(1, True)
+    single.forecast(1, False)
+    d = single.assimilate(xy, y)
+    assert diag[0, 0] == d["w_target"] and diag[0, 1] == d["beta"] and diag[0, 2] == 0
+    assert np.array_equal(batch.instances[0].get_state(), single.get_state())
