@@ -9,6 +9,7 @@
 #include <string>
 #include <vector>
 
+#include <cuda.h>
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/iewpf.h"
@@ -109,15 +110,18 @@ struct iewpf_ctx {
     int nnz = 0;
     double* d_d = nullptr;      // innovations [ne][Ny]
     double* d_Sd = nullptr;     // [ne][Ny]
+    // an analysis' diagnostics in one allocation: phi, c, gamma, zeta, alpha,
+    // neglogw [ne] each, then scal [4] (w_target, beta, c_bar)
+    double* d_diag = nullptr;
     double* d_phi = nullptr;
     double* d_c = nullptr;
     double* d_gamma = nullptr;
     double* d_zeta = nullptr;
     double* d_alpha = nullptr;
-    double* d_cstar = nullptr;
     double* d_neglogw = nullptr;
+    double* d_scal = nullptr;
+    double* d_cstar = nullptr;
     double* d_coef = nullptr;   // [ne][2] (a_i, length scale)
-    double* d_scal = nullptr;   // [4] (c_bar, beta)
     double* d_partial = nullptr;
     int dots_blk = 0;
     float* d_r = nullptr;       // posterior coarse field [ne][N_R]
@@ -131,7 +135,8 @@ struct iewpf_ctx {
     // pinned staging
     int* h_flag = nullptr;
     int* h_maxsub = nullptr;
-    double* h_scal = nullptr;
+    double* h_diag = nullptr;      // host copy of d_diag
+    cudaEvent_t ev_user = nullptr;  // orders a caller's stream before a state copy
     // counters
     uint32_t step = 0, cycle = 0;
     int64_t launches = 0;    // kernels launched
@@ -866,7 +871,7 @@ int iewpf_create(const iewpf_params_t* params, const double* mooring_xy, iewpf_c
         return bail(rc);
     if (cudaMallocHost((void**)&ctx->h_flag, sizeof(int)) != cudaSuccess ||
         cudaMallocHost((void**)&ctx->h_maxsub, sizeof(int)) != cudaSuccess ||
-        cudaMallocHost((void**)&ctx->h_scal, 4 * sizeof(double)) != cudaSuccess ||
+        cudaMallocHost((void**)&ctx->h_diag, (6 * (size_t)P.n_particles + 4) * sizeof(double)) != cudaSuccess ||
         cudaMallocHost((void**)&ctx->h_step, sizeof(uint32_t)) != cudaSuccess ||
         cudaMallocHost((void**)&ctx->h_iters, sizeof(unsigned int)) != cudaSuccess)
         return bail(IEWPF_ENOMEM);
@@ -903,15 +908,15 @@ int iewpf_create(const iewpf_params_t* params, const double* mooring_xy, iewpf_c
         (rc = dalloc(ctx, &ctx->d_L, ny * ny)) || (rc = dalloc(ctx, &ctx->d_colptr, ny + 1)) ||
         (rc = dalloc(ctx, &ctx->d_rowidx, ny * (ny - 1) / 2 + ny)) || (rc = dalloc(ctx, &ctx->d_d, ne * ny)) ||
         (rc = dalloc(ctx, &ctx->d_rdiag, ny)) || (rc = dalloc(ctx, &ctx->d_plan, solve_plan_ints((int)ny))) ||
-        (rc = dalloc(ctx, &ctx->d_Sd, ne * ny)) || (rc = dalloc(ctx, &ctx->d_phi, ne)) ||
-        (rc = dalloc(ctx, &ctx->d_c, ne)) || (rc = dalloc(ctx, &ctx->d_gamma, ne)) ||
-        (rc = dalloc(ctx, &ctx->d_zeta, ne)) || (rc = dalloc(ctx, &ctx->d_alpha, ne)) ||
-        (rc = dalloc(ctx, &ctx->d_cstar, ne)) || (rc = dalloc(ctx, &ctx->d_neglogw, ne)) ||
-        (rc = dalloc(ctx, &ctx->d_coef, 2 * ne)) || (rc = dalloc(ctx, &ctx->d_scal, 4)) ||
+        (rc = dalloc(ctx, &ctx->d_Sd, ne * ny)) || (rc = dalloc(ctx, &ctx->d_diag, 6 * ne + 4)) ||
+        (rc = dalloc(ctx, &ctx->d_cstar, ne)) || (rc = dalloc(ctx, &ctx->d_coef, 2 * ne)) ||
         (rc = dalloc(ctx, &ctx->d_partial, ne * ctx->dots_blk * 3)) ||
         (rc = dalloc(ctx, &ctx->d_r, ne * (size_t)ctx->NR)) || (rc = dalloc(ctx, &ctx->d_xi, ne * (size_t)ctx->NR)) ||
         (rc = dalloc(ctx, &ctx->d_soar, ne * (size_t)ctx->NR)))
         return bail(rc);
+    double** const diag[] = {&ctx->d_phi, &ctx->d_c, &ctx->d_gamma, &ctx->d_zeta, &ctx->d_alpha, &ctx->d_neglogw,
+                             &ctx->d_scal};
+    for (int i = 0; i < 7; ++i) *diag[i] = ctx->d_diag + i * ne;
     if (P.n_drifters_max > 0 && (rc = dalloc(ctx, &ctx->d_xy, ne * 2 * (size_t)P.n_drifters_max)))
         return bail(rc);
     if (P.obs_kind == IEWPF_OBS_MOORING && nobs > 0) {
@@ -991,14 +996,15 @@ int iewpf_destroy(iewpf_ctx_t* ctx)
                     ctx->d_wtab, ctx->d_K32, ctx->d_K64, ctx->d_M49, ctx->d_xy, ctx->d_obs_xy, ctx->d_obs_y,
                     ctx->d_cell, ctx->d_block0, ctx->d_border, ctx->d_blevel, ctx->d_perm_u, ctx->d_cell_perm, ctx->d_xs,
                     ctx->d_tile_cnt, ctx->d_tile_obs, ctx->d_L, ctx->d_colptr,
-                    ctx->d_rowidx, ctx->d_rdiag, ctx->d_plan, ctx->d_Lr, ctx->d_Lc, ctx->d_stream, ctx->d_d, ctx->d_Sd, ctx->d_phi, ctx->d_c, ctx->d_gamma, ctx->d_zeta,
-                    ctx->d_alpha, ctx->d_cstar, ctx->d_neglogw, ctx->d_coef, ctx->d_scal, ctx->d_partial,
+                    ctx->d_rowidx, ctx->d_rdiag, ctx->d_plan, ctx->d_Lr, ctx->d_Lc, ctx->d_stream, ctx->d_d, ctx->d_Sd, ctx->d_diag,
+                    ctx->d_cstar, ctx->d_coef, ctx->d_partial,
                     ctx->d_r, ctx->d_xi, ctx->d_soar};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (ctx->h_flag) cudaFreeHost(ctx->h_flag);
     if (ctx->h_maxsub) cudaFreeHost(ctx->h_maxsub);
-    if (ctx->h_scal) cudaFreeHost(ctx->h_scal);
+    if (ctx->h_diag) cudaFreeHost(ctx->h_diag);
+    if (ctx->ev_user) cudaEventDestroy(ctx->ev_user);
     if (ctx->h_step) cudaFreeHost(ctx->h_step);
     if (ctx->h_iters) cudaFreeHost(ctx->h_iters);
     for (auto& fg : ctx->fgraphs) cudaGraphExecDestroy(fg.exec);
@@ -1010,6 +1016,31 @@ int iewpf_destroy(iewpf_ctx_t* ctx)
     return IEWPF_OK;
 }
 
+// whether a kernel may take [p, p + bytes): device memory of device dev, inside
+// one allocation, float-aligned.  Anything else (another device's memory,
+// managed memory, a range that cudaMemcpy would refuse) is left to cudaMemcpy
+static bool device_range(const void* p, size_t bytes, int dev)
+{
+    static const auto range = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+            r != cudaDriverEntryPointSuccess)
+            f = nullptr;
+        return reinterpret_cast<CUresult(CUDAAPI*)(CUdeviceptr*, size_t*, CUdeviceptr)>(f);
+    }();
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+    return a.type == cudaMemoryTypeDevice && a.device == dev && at % sizeof(float) == 0 && range &&
+           range(&base, &size, at) == CUDA_SUCCESS && at - base + bytes <= size;
+}
+
 static int copy_state(iewpf_ctx_t* ctx, float* host_or_dev, int on_device, void* stream, bool in)
 {
     if (!ctx) return IEWPF_EINVAL;
@@ -1018,17 +1049,15 @@ static int copy_state(iewpf_ctx_t* ctx, float* host_or_dev, int on_device, void*
     CK(cudaSetDevice(ctx->dev));
     cudaStream_t user = (cudaStream_t)stream;
     if (user) {
-        cudaEvent_t ev;
-        CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-        CK(cudaEventRecord(ev, user));
-        CK(cudaStreamWaitEvent(ctx->st, ev, 0));
-        CK(cudaEventDestroy(ev));
+        if (!ctx->ev_user) CK(cudaEventCreateWithFlags(&ctx->ev_user, cudaEventDisableTiming));
+        CK(cudaEventRecord(ctx->ev_user, user));
+        CK(cudaStreamWaitEvent(ctx->st, ctx->ev_user, 0));
     }
     const size_t per = 3 * (size_t)ctx->plane;
-    std::vector<int> par(ctx->G.ne);
-    if (!in) {
-        CK(cudaMemcpyAsync(par.data(), ctx->par, sizeof(int) * par.size(), cudaMemcpyDeviceToHost, ctx->st));
+    if (on_device && device_range(host_or_dev, sizeof(float) * per * ctx->G.ne, ctx->dev)) {
+        KL(1, launch_state_copy(in, host_or_dev, ctx->buf[0], ctx->buf[1], ctx->par, ctx->G, ctx->st));
         CK(cudaStreamSynchronize(ctx->st));
+        return IEWPF_OK;
     }
     const cudaMemcpyKind kind = in ? (on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice)
                                    : (on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost);
@@ -1036,6 +1065,9 @@ static int copy_state(iewpf_ctx_t* ctx, float* host_or_dev, int on_device, void*
         CK(cudaMemcpyAsync(ctx->buf[0], host_or_dev, sizeof(float) * per * ctx->G.ne, kind, ctx->st));
         CK(cudaMemsetAsync(ctx->par, 0, sizeof(int) * ctx->G.ne, ctx->st));
     } else {
+        std::vector<int> par(ctx->G.ne);
+        CK(cudaMemcpyAsync(par.data(), ctx->par, sizeof(int) * par.size(), cudaMemcpyDeviceToHost, ctx->st));
+        CK(cudaStreamSynchronize(ctx->st));
         // contiguous runs of particles that live in the same buffer
         int p = 0;
         while (p < ctx->G.ne) {
@@ -1146,18 +1178,19 @@ int iewpf_assimilate(iewpf_ctx_t* ctx, const iewpf_obs_t* obs, iewpf_diag_t* dia
     KL(qhalf_launches(A), launch_qhalf(A, ctx->G, ctx->C, ctx->st));
     ctx->cfl_ready = true;
     // diagnostics
-    CK(cudaMemcpyAsync(ctx->h_scal, ctx->d_scal, 3 * sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
-    if (diag) {
-        double* dst[] = {diag->phi, diag->c, diag->gamma, diag->zeta, diag->alpha, diag->neglogw};
-        double* src[] = {ctx->d_phi, ctx->d_c, ctx->d_gamma, ctx->d_zeta, ctx->d_alpha, ctx->d_neglogw};
-        for (int i = 0; i < 6; ++i)
-            if (dst[i]) CK(cudaMemcpyAsync(dst[i], src[i], sizeof(double) * ne, cudaMemcpyDeviceToHost, ctx->st));
-    }
+    // (one copy to pinned memory: a copy per array into the caller's pageable
+    // memory waits for each)
+    if (diag) CK(cudaMemcpyAsync(ctx->h_diag, ctx->d_diag, sizeof(double) * (6 * (size_t)ne + 4), cudaMemcpyDeviceToHost,
+                                 ctx->st));
     rc = read_flags(ctx);
     if (diag) {
-        diag->w_target = ctx->h_scal[0];
-        diag->beta = ctx->h_scal[1];
-        diag->c_bar = ctx->h_scal[2];
+        double* dst[] = {diag->phi, diag->c, diag->gamma, diag->zeta, diag->alpha, diag->neglogw};
+        for (int i = 0; i < 6; ++i)
+            if (dst[i]) std::memcpy(dst[i], ctx->h_diag + (size_t)i * ne, sizeof(double) * ne);
+        const double* scal = ctx->h_diag + 6 * (size_t)ne;
+        diag->w_target = scal[0];
+        diag->beta = scal[1];
+        diag->c_bar = scal[2];
     }
     ctx->cycle++;
     return rc;

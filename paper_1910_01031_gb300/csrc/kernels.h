@@ -36,6 +36,8 @@ cudaError_t launch_drift(const float* b0, const float* b1, const int* par, const
                          const int* s_dev = nullptr);
 cudaError_t launch_drift_errors(const double* xy, const double* truth, int ne, int nd, double* E, double* RMSE,
                                 cudaStream_t st);
+// the ensemble from (in) or to a device array ext; in resets par
+cudaError_t launch_state_copy(bool in, float* ext, float* b0, float* b1, int* par, const Grid& G, cudaStream_t st);
 cudaError_t launch_nonfinite(const float* b0, const float* b1, const int* par, const Grid& G, int* flag,
                              cudaStream_t st);
 

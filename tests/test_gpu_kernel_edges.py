@@ -196,3 +196,27 @@ def test_factor_by_levels_equals_column_by_column(n, spread):
     d = single.assimilate(xy, y)
     assert diag[0, 0] == d["w_target"] and diag[0, 1] == d["beta"] and diag[0, 2] == 0
     assert np.array_equal(batch.instances[0].get_state(), single.get_state())
+
+
+@pytest.mark.parametrize("nx,ny,offset", [(64, 64, 0), (64, 64, 1), (64, 64, 4), (45, 47, 0), (50, 46, 2), (150, 141, 3)])
+def test_device_state_copies(nx, ny, offset):
+    """States in and out of device memory by 16 bytes or by single values (planes of any remainder, arrays off
+    their alignment), particles in either buffer: the copies through host memory, bit for bit."""
+    import torch
+    cfg = synth.Config("edge", nx, ny, n_particles=5)
+    U32, _ = start_state(cfg, 5)
+    U32[3] *= np.float32(1.5)                # other wave speeds: other numbers of scheme steps
+    a, b = ensemble(cfg), ensemble(cfg)
+    flat = torch.zeros(offset + U32.size + 8, dtype=torch.float32, device="cuda")
+    view = flat[offset:offset + U32.size].view(*U32.shape)
+    view.copy_(torch.from_numpy(U32))
+    a.set_state(view)
+    b.set_state(U32)
+    for steps in (0, 1, 1):
+        if steps:
+            a.forecast(steps, True)
+            b.forecast(steps, True)
+        flat.fill_(-1.0)
+        a.get_state(view)
+        assert np.array_equal(view.cpu().numpy(), b.get_state())
+        assert bool((flat[:offset] == -1).all()) and bool((flat[offset + U32.size:] == -1).all())
