@@ -160,6 +160,13 @@ __global__ void b_par(BatchDev B)
     }
 }
 
+// a / b of non-negative numbers, in 32 bits where both fit (64-bit division is
+// a few times the instructions)
+__device__ __forceinline__ long long quotient(long long a, long long b)
+{
+    return ((a | b) >> 32) == 0 ? (long long)((uint32_t)a / (uint32_t)b) : a / b;
+}
+
 // model error (coarse field from Philox) and analysis update (posterior coarse
 // field plus the pull), staged:
 // coarse normals per Philox block, SOAR per coarse point, fine tiles
@@ -170,8 +177,8 @@ __global__ void b_normals(BatchDev B)
         const int i = find_inst(pre, B.n, q);
         const BInst& I = B.inst[i];
         const long long nq = (I.NR + 3) / 4, r = q - pre[i];
-        const int p = (int)(r / nq);
-        qhalf::normals_block(seed_key(I.seed), (uint32_t)p, *I.step_ctr, I.stream_base, (uint32_t)(r % nq), I.NR,
+        const int p = (int)quotient(r, nq);
+        qhalf::normals_block(seed_key(I.seed), (uint32_t)p, *I.step_ctr, I.stream_base, (uint32_t)(r - p * nq), I.NR,
                              I.xi + (long long)p * I.NR);
     }
 }
@@ -184,11 +191,11 @@ __global__ void b_soar(BatchDev B)
         const int i = find_inst(pre, B.n, q);
         const BInst& I = B.inst[i];
         const long long r = q - pre[i];
-        const long long p = r / I.NR, m = r % I.NR;
         const Grid G = I.G;
         const Coarse C = I.C;
-        I.soar[p * I.NR + m] = qhalf::soar_point((POSTERIOR ? I.r : I.xi) + p * I.NR, I.wtab, C, G,
-                                                 (int)(m % C.nRx), (int)(m / C.nRx));
+        const long long p = quotient(r, I.NR);
+        const int m = (int)(r - p * I.NR), bm = m / C.nRx;
+        I.soar[r] = qhalf::soar_point((POSTERIOR ? I.r : I.xi) + p * I.NR, I.wtab, C, G, m - bm * C.nRx, bm);
     }
 }
 
@@ -347,8 +354,9 @@ __global__ void b_form_r(BatchDev B)
         const int i = find_inst(pre, B.n, q);
         const BInst& I = B.inst[i];
         const long long nq = (I.NR + 3) / 4, r = q - pre[i];
+        const int p = (int)quotient(r, nq);
         ana::form_r_block(I.seed, *I.cycle, I.stream_base + 1, I.stream_base + 2, (int)I.NR, I.coef, I.scal, I.alpha,
-                          I.r, (int)(r / nq), (int)(r % nq));
+                          I.r, p, (int)(r - p * nq));
     }
 }
 

@@ -20,16 +20,44 @@ __global__ void coarse_normals_kernel(QhalfArgs A, long long NR)
     qhalf::normals_block(seed_key(A.seed), (uint32_t)p, t, A.stream, (uint32_t)q, NR, A.xi_buf + (long long)p * NR);
 }
 
-// Q_SOAR^{1/2} of every coarse point of every particle
-__global__ void coarse_soar_kernel(const float* __restrict__ src, const float* __restrict__ wtab, Grid G, Coarse C,
-                                   float* __restrict__ out)
+// Q_SOAR^{1/2} of every coarse point of every particle (blockIdx.z).  Bound by
+// instructions: the points two and more from the periodic seam in groups of
+// SOAR_ROWS rows, a warp along the columns, the others (whose neighbours and
+// distances take index arithmetic) densely packed in CTAs of their own, the
+// rows of blocks from inner_y on.  A point per thread with 64-bit divisions for
+// its place, the seam's points among the others: 279 us for 341^2 coarse points
+// x 256, now 106; 171^2 x 100: 38, now 18.
+__global__ void __launch_bounds__(256)
+coarse_soar_kernel(const float* __restrict__ src, const float* __restrict__ wtab, Grid G, Coarse C,
+                   float* __restrict__ out, int inner_y)
 {
     const long long NR = (long long)C.nRx * C.nRy;
-    const long long m = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= NR) return;
-    const int p = blockIdx.y;
-    out[(long long)p * NR + m] =
-        qhalf::soar_point(src + (long long)p * NR, wtab, C, G, (int)(m % C.nRx), (int)(m / C.nRx));
+    const float* __restrict__ s = src + blockIdx.z * NR;
+    float* __restrict__ o = out + blockIdx.z * NR;
+    if ((int)blockIdx.y < inner_y) {
+        const int am = 2 + 32 * blockIdx.x + (threadIdx.x & 31);
+        const int bm = 2 + qhalf::SOAR_ROWS * (8 * blockIdx.y + (threadIdx.x >> 5));
+        if (am >= C.nRx - 2 || bm >= C.nRy - 2) return;
+        if (bm + qhalf::SOAR_ROWS <= C.nRy - 2) {
+            qhalf::soar_rows(s, wtab, C, am, bm, o);
+        } else {
+            for (int b = bm; b < C.nRy - 2; ++b) o[b * C.nRx + am] = qhalf::soar_point(s, wtab, C, G, am, b);
+        }
+        return;
+    }
+    const int e = (int)(((blockIdx.y - inner_y) * gridDim.x + blockIdx.x) * 256 + threadIdx.x);
+    int am, bm;
+    if (e < 4 * C.nRy) {                 // the first and last two columns
+        const int c = e / C.nRy;
+        am = c < 2 ? c : C.nRx - 4 + c;
+        bm = e - c * C.nRy;
+    } else {                             // the rest of the first and last two rows
+        const int f = e - 4 * C.nRy, c = f / (C.nRx - 4);
+        if (c >= 4) return;
+        bm = c < 2 ? c : C.nRy - 4 + c;
+        am = 2 + f - c * (C.nRx - 4);
+    }
+    o[bm * C.nRx + am] = qhalf::soar_point(s, wtab, C, G, am, bm);
 }
 
 // model error and analysis update on FINE_TX x FINE_TY tiles (the analysis
@@ -84,7 +112,10 @@ cudaError_t launch_qhalf(const QhalfArgs& A, const Grid& G, const Coarse& C, cud
         coarse_normals_kernel<<<dim3((unsigned)((nq + 255) / 256), G.ne), 256, 0, st>>>(A, NR);
         src = A.xi_buf;
     }
-    coarse_soar_kernel<<<dim3((unsigned)((NR + 255) / 256), G.ne), 256, 0, st>>>(src, A.wtab, G, C, A.soar_buf);
+    const int bx = (C.nRx - 4 + 31) / 32, rows = 8 * qhalf::SOAR_ROWS, inner_y = (C.nRy - 4 + rows - 1) / rows;
+    const int seam = (4 * C.nRy + 4 * (C.nRx - 4) + 255) / 256;
+    coarse_soar_kernel<<<dim3(bx, inner_y + (seam + bx - 1) / bx, G.ne), 256, 0, st>>>(src, A.wtab, G, C, A.soar_buf,
+                                                                                     inner_y);
     const int tiles = ((G.nx + FINE_TX - 1) / FINE_TX) * ((G.ny + FINE_TY - 1) / FINE_TY);
     const int parts = qhalf::fine_choice(
         [&](int n) { return (long long)tiles * ((G.ne + n - 1) / n); }, tc::sm_count());

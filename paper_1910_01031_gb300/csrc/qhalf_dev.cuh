@@ -72,6 +72,37 @@ __device__ __forceinline__ float soar_point(const float* __restrict__ src, const
     return acc;
 }
 
+// points (am, bm0 + r), r < SOAR_ROWS, all two and more away from the seam:
+// each row of five neighbours is loaded once for the points it enters; the
+// sums of soar_point, term by term
+constexpr int SOAR_ROWS = 4;
+__device__ __forceinline__ void soar_rows(const float* __restrict__ src, const float* __restrict__ wtab, const Coarse& C,
+                                          int am, int bm0, float* __restrict__ out)
+{
+    float w[3][3], acc[SOAR_ROWS];
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) w[b][a] = __ldg(wtab + C.c * b * C.tab + C.c * a);
+#pragma unroll
+    for (int j = 0; j < SOAR_ROWS + 4; ++j) {
+        const float* __restrict__ row = src + (bm0 - 2 + j) * C.nRx + am;
+        float v[5];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) v[k] = row[k - 2];
+#pragma unroll
+        for (int r = 0; r < SOAR_ROWS; ++r) {
+            const int db = j - 2 - r;
+            if (db < -2 || db > 2) continue;
+            if (db == -2) acc[r] = 0.0f;
+#pragma unroll
+            for (int k = 0; k < 5; ++k) acc[r] = fmaf(w[db < 0 ? -db : db][k < 2 ? 2 - k : k - 2], v[k], acc[r]);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < SOAR_ROWS; ++r) out[(bm0 + r) * C.nRx + am] = acc[r];
+}
+
 // The fine stage: a warp marches down a strip of 32 columns of PB particles
 // at once, one column per lane, with no shared memory between lanes and no
 // barriers: the four coarse rows around the current row, interpolated in x at

@@ -220,3 +220,16 @@ def test_device_state_copies(nx, ny, offset):
         a.get_state(view)
         assert np.array_equal(view.cpu().numpy(), b.get_state())
         assert bool((flat[:offset] == -1).all()) and bool((flat[offset + U32.size:] == -1).all())
+
+
+@pytest.mark.parametrize("nx,ny,c", [(16, 16, 1), (17, 18, 1), (36, 37, 1), (37, 67, 1), (68, 39, 1), (48, 54, 3), (107, 51, 3)])
+def test_coarse_correlation_over_row_groups(nx, ny, c):
+    """The 5 x 5 SOAR sums in groups of four rows with the periodic seam apart: coarse grids of one column of
+    blocks and more, every remainder of rows, one model step with model error against the oracle at 1e-5."""
+    cfg = synth.Config("edge", nx, ny, n_particles=3, c_omega=c)
+    ens, P = ensemble(cfg), oracle_problem(cfg)
+    U32, U64 = start_state(cfg, 3)
+    ens.set_state(U32)
+    ens.forecast(1, True)
+    ref, _, _ = O.forecast(P, U64, 1, True, t0=0)
+    assert rel_l2(ens.get_state(), ref) <= 1e-5
