@@ -969,7 +969,7 @@ __device__ __forceinline__ void rand_dots_cta(uint64_t seed, uint32_t t, uint32_
                                               double* __restrict__ partial, int nblk, int p, int bx)
 {
     const uint2 key = seed_key(seed);
-    const int nq = (NR + 3) / 4;
+    const int nq = NR / 4;                           // whole blocks
     double px = 1.0, pn = 1.0;                       // products of the u_a of xi and of nu~
     double tx = 0.0, tn = 0.0, tc = 0.0;             // terms of the last, partial block
     float cs = 0.0f, ce = 0.0f;                      // cross product: sum and its rounding errors
@@ -977,32 +977,36 @@ __device__ __forceinline__ void rand_dots_cta(uint64_t seed, uint32_t t, uint32_
     for (int b = bx * DOT_THREADS + threadIdx.x; b < nq; b += nblk * DOT_THREADS) {
         const uint4 wx = philox4x32_10(make_uint4((uint32_t)b, (uint32_t)p, t, s_xi), key);
         const uint4 wn = philox4x32_10(make_uint4((uint32_t)b, (uint32_t)p, t, s_nu), key);
-        if (4 * b + 3 < NR) {
-            px *= uniform64(wx.x) * uniform64(wx.z);
-            pn *= uniform64(wn.x) * uniform64(wn.z);
-            const uint32_t xa[2] = {wx.x, wx.z}, xb[2] = {wx.y, wx.w}, na[2] = {wn.x, wn.z}, nb[2] = {wn.y, wn.w};
+        px *= uniform64(wx.x) * uniform64(wx.z);
+        pn *= uniform64(wn.x) * uniform64(wn.z);
+        const uint32_t xa[2] = {wx.x, wx.z}, xb[2] = {wx.y, wx.w}, na[2] = {wn.x, wn.z}, nb[2] = {wn.y, wn.w};
 #pragma unroll
-            for (int l = 0; l < 2; ++l) {
-                const float r = sqrtf(4.0f * log_uniform32(xa[l]) * log_uniform32(na[l]));
-                const float c = cospif((float)(int)(nb[l] - xb[l]) * 0x1p-31f);
-                const float v = r * c, ve = fmaf(r, c, -v);
-                const float s = cs + v, bb = s - cs;
-                ce += ((cs - (s - bb)) + (v - bb)) + ve;
-                cs = s;
-            }
-        } else {
-            double x[4], v[4];
-            box_muller64(wx.x, wx.y, x[0], x[1]);
-            box_muller64(wx.z, wx.w, x[2], x[3]);
-            box_muller64(wn.x, wn.y, v[0], v[1]);
-            box_muller64(wn.z, wn.w, v[2], v[3]);
+        for (int l = 0; l < 2; ++l) {
+            const float r = sqrtf(4.0f * log_uniform32(xa[l]) * log_uniform32(na[l]));
+            const float c = cospif((float)(int)(nb[l] - xb[l]) * 0x1p-31f);
+            const float v = r * c, ve = fmaf(r, c, -v);
+            const float s = cs + v, bb = s - cs;
+            ce += ((cs - (s - bb)) + (v - bb)) + ve;
+            cs = s;
+        }
+    }
+    // a last block of 1 to 3 normals: its pairs in FP64, one per lane of one warp
+    // (pair lane / 2 of xi or, odd lanes, of nu~; one after the other in a thread
+    // they were half of the kernel at 64 x 64)
+    if (4 * nq < NR && bx == nblk - 1 && threadIdx.x >= DOT_THREADS - 32) {
+        const int lane = threadIdx.x & 31;
+        double z[2] = {0.0, 0.0};
+        if (lane < 4) {
+            const uint4 w = philox4x32_10(make_uint4((uint32_t)nq, (uint32_t)p, t, lane & 1 ? s_nu : s_xi), key);
+            box_muller64(lane & 2 ? w.z : w.x, lane & 2 ? w.w : w.y, z[0], z[1]);
+        }
 #pragma unroll
-            for (int l = 0; l < 4; ++l) {
-                if (4 * b + l < NR) {
-                    tx = fma(x[l], x[l], tx);
-                    tn = fma(v[l], v[l], tn);
-                    tc = fma(v[l], x[l], tc);
-                }
+        for (int l = 0; l < 3; ++l) {
+            const double x = __shfl_sync(0xffffffffu, z[l & 1], l & 2), v = __shfl_sync(0xffffffffu, z[l & 1], (l & 2) + 1);
+            if (lane == 0 && 4 * nq + l < NR) {
+                tx = fma(x, x, tx);
+                tn = fma(v, v, tn);
+                tc = fma(v, x, tc);
             }
         }
     }
