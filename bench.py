@@ -47,10 +47,11 @@ UNIT = "particle*cell*step/s"
 BYTES_PER_CELL_STEP = 24          # read (eta, hu, hv) + write (eta, hu, hv), float32
 # FP32 operations of one scheme step per cell (adds, multiplies and fused
 # multiply-adds, one each; no halo), counted from the kernel's arithmetic
-SCHEME_OPS_PER_CELL_STEP = 260
-# issue slots per cell and scheme step measured by ncu at 512^2 x 100
-# (smsp__inst_executed.sum x 32 / cells), per stepper kind
-ISSUE_PER_CELL_STEP = {1: 524.3, 2: 363.3}
+SCHEME_OPS_PER_CELL_STEP = 216
+# instructions per cell and scheme step measured by ncu at 512^2 x 100
+# (smsp__inst_executed.sum x 32 / cells), per stepper kind; of the paired
+# kind's, 125 are packed and take two dispatch slots each
+ISSUE_PER_CELL_STEP = {1: 451.0, 2: 337.0}
 WORKLOAD = "iewpf_cycle_1024x1024_ne1000_1521moorings"
 LEGS = ("drifters", "coupled", "batched", "batched_small", "surrogate", "one_stage", "rank_histogram")
 
@@ -227,8 +228,8 @@ def scheme_step_roofline(ens, cfg, stream, local, n=13):
     shape = ens.stepper()
     return {"bound": "hbm", "achieved": round(achieved_gbs, 1), "peak": hbm_peak, "unit": "GB/s",
             "frac": round(achieved_gbs / hbm_peak, 4), "traffic": traffic,
-            "kernel": "%s (SSP-RK2 scheme step, register march), shape (kind, nc, rows, warps) = %s"
-                      % ("rk2_march2_kernel" if shape[0] == 2 else "rk2_march_kernel", shape,),
+            "kernel": "rk2_march_kernel (SSP-RK2 scheme step, register march), shape (kind, nc, rows, warps) = %s"
+                      % (shape,),
             "per_launch_ms": round(launch_s * 1e3, 4), "cells_per_launch": cells,
             "fp32": {"achieved": round(ops, 2), "peak": round(fp32_ops_peak, 1), "unit": "Top/s",
                      "frac": round(ops / fp32_ops_peak, 4), "ops_per_cell_step": SCHEME_OPS_PER_CELL_STEP},
