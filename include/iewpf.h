@@ -382,6 +382,13 @@ IEWPF_API int iewpf_local_block(const iewpf_ctx_t* ctx, double* M);
  * centre outside the grid). */
 IEWPF_API int iewpf_block_levels(const int* block0, int nobs, int nRx, int nRy, int* level);
 
+/* Particles that share a CTA in the triangular solves S d of a fixed layout
+ * of n = 2 n_obs unknowns (256 moorings and more; n_particles particles on a
+ * device of `sms` SMs): 8 or 4, or 1 (a warp per particle, as in smaller
+ * layouts).  The results do not depend on it.  Host arithmetic only (no
+ * device).  Errors: EINVAL (a number < 1, NULL particles). */
+IEWPF_API int iewpf_solve_group(int n, int n_particles, int sms, int* particles);
+
 /* Add Q^{1/2} x to every particle for coarse fields x ([N_e][N_R] float32,
  * host), the operator of eq. covarianceOperatorsDef (testing aid).
  * Errors: EINVAL (NULL x), ECUDA. */

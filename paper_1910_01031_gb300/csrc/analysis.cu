@@ -15,6 +15,8 @@ namespace {
 constexpr int kCholSmem = 212 * 1024;
 // dynamic shared memory of a CTA of the grouped sweeps at most
 constexpr int kSolveGroupSmem = 224 * 1024;
+static_assert(ana::solve_group_smem<4>((int)(kSolveSmemBytes / sizeof(double))) > kSolveGroupSmem,
+              "a layout that fits a group fits a warp");
 
 __global__ void obs_cells_kernel(const double* __restrict__ xy, int nobs, Grid G, Coarse C, double dx, double dy,
                                  int* __restrict__ cell, int* __restrict__ block0)
@@ -320,26 +322,36 @@ cudaError_t launch_cholesky(double* M, int n, int* colptr, int* rowidx, int* fla
     return cudaGetLastError();
 }
 
+// Several particles per CTA where their vectors fit its shared memory (n <=
+// 6140 for 4, 3064 for 8) and that takes at most 3 / 2 as many waves of CTAs as
+// a warp each does (a wave of 1521 coupled moorings, n = 3042: 3.4 ms against
+// 5.5), and of 4 and 8 the one with fewer waves (4 at a tie: 5350 against 5624 us
+// per analysis of 100 particles; of 1000, 8 takes one wave and 13.2 ms, 4 two
+// and 16.0, a warp each 15.4).  Where a group fits, a warp's vector does too
+// (solve_smem_kernel), so that kernel's shared memory sets the waves compared
+// with.
+int solve_group(int n, int ne, int sms)
+{
+    // 16 warps of these kernels are resident per SM
+    auto waves = [&](int P, size_t smem) {
+        const size_t resident = std::min((size_t)16 / P, (size_t)(228 * 1024) / (smem + 1024));
+        return ((size_t)(ne + P - 1) / P + sms * resident - 1) / (sms * resident);
+    };
+    const size_t s4 = ana::solve_group_smem<4>(n), s8 = ana::solve_group_smem<8>(n);
+    if (s4 > kSolveGroupSmem) return 1;
+    const size_t w1 = waves(1, (size_t)n * sizeof(double)), w4 = waves(4, s4);
+    const size_t w8 = s8 <= kSolveGroupSmem ? waves(8, s8) : w4 + 1;
+    if (2 * std::min(w4, w8) > 3 * w1) return 1;
+    return w4 <= w8 ? 4 : 8;
+}
+
 cudaError_t launch_solve(const double* L, const int* colptr, const int* rowidx, const double* rdiag, const int* plan,
                          int n, const double* d, double* Sd, double* phi, int ne, cudaStream_t st, const int* perm,
                          double* scratch, const double* Lr, const double* Lc, const void* stream, int nnz)
 {
     if ((perm && !scratch) || (!Lr != !Lc)) return cudaErrorInvalidValue;
     if (ne <= 0) return cudaSuccess;
-    // Several particles per CTA where that takes at most 3 / 2 as many waves of
-    // CTAs as a warp each does (a wave of 1521 coupled moorings, n = 3042: 3.4 ms
-    // against 5.5), and of 4 and 8 the one with fewer waves (4 at a tie: 5350
-    // against 5624 us per analysis of 100 particles; of 1000, 8 takes one wave
-    // and 13.2 ms, 4 two and 16.0, a warp each 15.4)
     if (stream && n > 0) {
-        const int sms = tc::sm_count();
-        auto waves = [&](int P, size_t smem) {
-            const size_t resident = std::min((size_t)16 / P, (size_t)(228 * 1024) / (smem + 1024));
-            return resident ? ((size_t)(ne + P - 1) / P + sms * resident - 1) / (sms * resident) : (size_t)1 << 30;
-        };
-        auto group_waves = [&](int P, size_t smem) { return smem <= kSolveGroupSmem ? waves(P, smem) : (size_t)1 << 30; };
-        const size_t w1 = waves(1, (size_t)n * sizeof(double)), w4 = group_waves(4, ana::solve_group_smem<4>(n)),
-                     w8 = group_waves(8, ana::solve_group_smem<8>(n));
         auto group = [&](auto Pc) {
             constexpr int P = decltype(Pc)::value;
             cudaError_t e = tc::smem_attr_once<solve_group_kernel<P>>(kSolveGroupSmem);
@@ -348,8 +360,9 @@ cudaError_t launch_solve(const double* L, const int* colptr, const int* rowidx, 
                                                                                                 phi, ne, perm);
             return cudaGetLastError();
         };
-        if (2 * std::min(w4, w8) <= 3 * w1)
-            return w4 <= w8 ? group(std::integral_constant<int, 4>()) : group(std::integral_constant<int, 8>());
+        const int P = solve_group(n, ne, tc::sm_count());
+        if (P == 4) return group(std::integral_constant<int, 4>());
+        if (P == 8) return group(std::integral_constant<int, 8>());
     }
     if (n > 0 && (size_t)n * sizeof(double) <= kSolveSmemBytes) {
         solve_smem_kernel<<<ne, 32, (size_t)n * sizeof(double), st>>>(L, colptr, rowidx, rdiag, plan, n, d, Sd, phi,

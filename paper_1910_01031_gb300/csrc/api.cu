@@ -1631,6 +1631,13 @@ int iewpf_local_block(const iewpf_ctx_t* ctx, double* M)
     return IEWPF_OK;
 }
 
+int iewpf_solve_group(int n, int n_particles, int sms, int* particles)
+{
+    if (n < 1 || n_particles < 1 || sms < 1 || !particles) return IEWPF_EINVAL;
+    *particles = solve_group(n, n_particles, sms);
+    return IEWPF_OK;
+}
+
 int iewpf_block_levels(const int* block0, int nobs, int nRx, int nRy, int* level)
 {
     if (nobs < 0 || nRx < 1 || nRy < 1 || (nobs > 0 && (!block0 || !level))) return IEWPF_EINVAL;

@@ -180,6 +180,10 @@ cudaError_t launch_solve(const double* L, const int* colptr, const int* rowidx, 
                          int n, const double* d, double* Sd, double* phi, int ne, cudaStream_t st,
                          const int* perm = nullptr, double* scratch = nullptr, const double* Lr = nullptr,
                          const double* Lc = nullptr, const void* stream = nullptr, int nnz = 0);
+// host: particles per CTA of the sweeps of a fixed layout with a stream (n
+// unknowns, ne particles, sms SMs): 8 or 4 (solve_group_kernel), or 1 (a warp
+// per particle)
+int solve_group(int n, int ne, int sms);
 // after launch_cholesky: the factor (nnz entries below the diagonal) in the
 // order of the sweeps, solve_stream_bytes(n, nnz) bytes
 size_t solve_stream_bytes(int n, int nnz);

@@ -26,7 +26,7 @@ EXPORTS = ["iewpf_create", "iewpf_destroy", "iewpf_set_state", "iewpf_get_state"
            "iewpf_last_nsub", "iewpf_last_error", "iewpf_philox_blocks", "iewpf_normals", "iewpf_weights",
            "iewpf_weights_one_stage", "iewpf_sir_weights", "iewpf_alpha_gamma", "iewpf_rank",
            "iewpf_batch_forecast", "iewpf_drifter_obs",
-           "iewpf_pull_stencil", "iewpf_local_block", "iewpf_block_levels", "iewpf_add_qhalf", "iewpf_sizes", "iewpf_stream",
+           "iewpf_pull_stencil", "iewpf_local_block", "iewpf_block_levels", "iewpf_solve_group", "iewpf_add_qhalf", "iewpf_sizes", "iewpf_stream",
            "iewpf_substeps", "iewpf_factor_info", "iewpf_launch_count", "iewpf_work", "iewpf_weights_noalloc", "iewpf_set_stepper", "iewpf_tune",
            "iewpf_get_stepper", "drifter_forecast_errors", "iewpf_batch_create", "iewpf_batch_destroy",
            "iewpf_batch_instance", "iewpf_batch_tune", "iewpf_batch_cycle", "iewpf_batch_stream",
@@ -157,6 +157,7 @@ def load(build_if_needed: bool = True):
     L.iewpf_surrogate_stream.argtypes = [_vp, c.POINTER(c.c_void_p)]
     L.iewpf_surrogate_loss_grad.argtypes = [_vp, _fp, _fp, c.c_int, _dp, _fp]
     L.iewpf_block_levels.argtypes = [_ip, c.c_int, c.c_int, c.c_int, _ip]
+    L.iewpf_solve_group.argtypes = [c.c_int, c.c_int, c.c_int, _ip]
     L.iewpf_surrogate_train.argtypes = [_vp, _vp, c.c_int, c.c_int, c.c_int, c.c_int, c.c_double, _dp]
     L.iewpf_surrogate_train_time.argtypes = [_vp, _dp]
     L.iewpf_set_surrogate.argtypes = [_vp, _vp, c.c_int]
@@ -714,6 +715,17 @@ def block_levels(block0, nRx, nRy):
     if rc != IEWPF_OK:
         raise IewpfError(rc, "block_levels")
     return out
+
+
+def solve_group(n, n_particles, sms=152):
+    """Particles that share a CTA in the triangular solves of a fixed layout
+    of n unknowns: 8, 4 or 1."""
+    L = load()
+    out = ctypes.c_int()
+    rc = L.iewpf_solve_group(int(n), int(n_particles), int(sms), ctypes.byref(out))
+    if rc != IEWPF_OK:
+        raise IewpfError(rc, "solve_group")
+    return out.value
 
 
 def alpha_gamma(gamma, cstar, N_psi):
