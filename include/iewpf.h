@@ -142,13 +142,15 @@ IEWPF_API int iewpf_destroy(iewpf_ctx_t* ctx);
 
 /* Copy the ensemble in ([N_e][3][ny][nx] float32; the state psi of Sec. 2,
  * fields (eta, hu, hv) of Sec. 3.1).  on_device: src is a device pointer
- * (copied on the context stream, after `stream` if given), else host
+ * (copied on the context stream, after the work queued on `stream`, NULL
+ * being the legacy default stream; the call returns when done), else host
  * memory.  Clears the CFL rates kept from the last update.
  * Errors: EINVAL (NULL pointer), ECUDA. */
 IEWPF_API int iewpf_set_state(iewpf_ctx_t* ctx, const float* src, int on_device, void* stream);
 
 /* Copy the ensemble out ([N_e][3][ny][nx] float32), to device memory when
- * on_device (ordered after the context's work and before `stream`), else to
+ * on_device (after the context's work and the work queued on `stream`, NULL
+ * being the legacy default stream; the call returns when done), else to
  * host memory.  Errors: EINVAL (NULL pointer), ECUDA. */
 IEWPF_API int iewpf_get_state(iewpf_ctx_t* ctx, float* dst, int on_device, void* stream);
 
@@ -559,10 +561,11 @@ IEWPF_API int iewpf_surrogate_inject_timeout(iewpf_surrogate_t* s, int n_evals);
 IEWPF_API int iewpf_surrogate_apply(iewpf_surrogate_t* s, const float* U, int n, float* Unext);
 /* The same on device memory: U and Unext (may be equal: in place) are
  * device pointers [n][3][ny][nx], borrowed; the work is ordered after the
- * work queued on `stream` (NULL: the call returns when done) and `stream`
- * waits for it.  Particles go through the network in chunks of 64.  With a
- * stream, a timeout of a bounded wait inside the tensor-core kernel
- * (IEWPF_ETIMEOUT) is reported by the next synchronous call. */
+ * work queued on `stream` (NULL: on the legacy default stream, and the call
+ * returns when done) and `stream` waits for it.  Particles go through the
+ * network in chunks of 64.  With a stream, a timeout of a bounded wait inside
+ * the tensor-core kernel (IEWPF_ETIMEOUT) is reported by the next synchronous
+ * call. */
 IEWPF_API int iewpf_surrogate_apply_device(iewpf_surrogate_t* s, const float* U, int n, float* Unext, void* stream);
 /* The surrogate's own CUDA stream.  Errors: EINVAL. */
 IEWPF_API int iewpf_surrogate_stream(const iewpf_surrogate_t* s, void** stream);

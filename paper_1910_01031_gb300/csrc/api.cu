@@ -1016,6 +1016,30 @@ int iewpf_destroy(iewpf_ctx_t* ctx)
     return IEWPF_OK;
 }
 
+// orders st after the work queued on the caller's stream, by the event ev; a
+// null stream is CUDA's legacy default stream, which a non-blocking st does not
+// wait for by itself.  It is left alone while a blocking stream is being
+// captured (its use would be an error and end the capture), and not waited for
+// when it is idle; the query may run beside another thread's capture.
+static cudaError_t wait_for(cudaStream_t user, cudaStream_t st, cudaEvent_t ev)
+{
+    if (!user) {
+        user = cudaStreamLegacy;
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        cudaStreamCaptureStatus capture;
+        cudaError_t e = cudaStreamIsCapturing(user, &capture);
+        const bool captured = e == cudaErrorStreamCaptureImplicit;
+        if (e == cudaSuccess) e = cudaStreamQuery(user);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (e == cudaErrorNotReady || captured) cudaGetLastError();
+        if (e == cudaSuccess || captured) return cudaSuccess;
+        if (e != cudaErrorNotReady) return e;
+    }
+    const cudaError_t e = cudaEventRecord(ev, user);
+    return e == cudaSuccess ? cudaStreamWaitEvent(st, ev, 0) : e;
+}
+
 // whether a kernel may take [p, p + bytes): device memory of device dev, inside
 // one allocation, float-aligned.  Anything else (another device's memory,
 // managed memory, a range that cudaMemcpy would refuse) is left to cudaMemcpy
@@ -1047,11 +1071,9 @@ static int copy_state(iewpf_ctx_t* ctx, float* host_or_dev, int on_device, void*
     if (in) ctx->cfl_ready = false;
     if (!host_or_dev) return fail(ctx, IEWPF_EINVAL, "null state pointer");
     CK(cudaSetDevice(ctx->dev));
-    cudaStream_t user = (cudaStream_t)stream;
-    if (user) {
+    if (stream || on_device) {
         if (!ctx->ev_user) CK(cudaEventCreateWithFlags(&ctx->ev_user, cudaEventDisableTiming));
-        CK(cudaEventRecord(ctx->ev_user, user));
-        CK(cudaStreamWaitEvent(ctx->st, ctx->ev_user, 0));
+        CK(wait_for((cudaStream_t)stream, ctx->st, ctx->ev_user));
     }
     const size_t per = 3 * (size_t)ctx->plane;
     if (on_device && device_range(host_or_dev, sizeof(float) * per * ctx->G.ne, ctx->dev)) {
@@ -2202,8 +2224,7 @@ int iewpf_surrogate_apply_device(iewpf_surrogate_t* s, const float* U, int n, fl
     cudaEvent_t ev;
     SCK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
     int rc = IEWPF_OK;
-    cudaError_t e = cudaSuccess;
-    if (user && (e = cudaEventRecord(ev, user)) == cudaSuccess) e = cudaStreamWaitEvent(s->st, ev, 0);
+    cudaError_t e = wait_for(user, s->st, ev);
     if (e == cudaSuccess && Unext != U) e = cudaMemcpyAsync(Unext, U, per * n * 4, cudaMemcpyDeviceToDevice, s->st);
     for (int p0 = 0; p0 < n && e == cudaSuccess && !rc; p0 += s->chunk) {
         const int nb = std::min(s->chunk, n - p0);
