@@ -9,6 +9,7 @@
 #pragma once
 #include "common.cuh"
 #include "kernels.h"
+#include "log_uniform.h"
 
 namespace iewpf {
 namespace ana {
@@ -942,12 +943,6 @@ __device__ __forceinline__ double uniform64(uint32_t a)
     return __hiloint2double(0x41300000, (int)a) - (0x1p20 - 0x1p-33);
 }
 
-// log u in FP32 to float precision over all of (0, 1), next to 1 as well (see box_muller32)
-__device__ __forceinline__ float log_uniform32(uint32_t a)
-{
-    return a < 0x80000000u ? logf(((float)a + 0.5f) * 0x1p-32f) : log1pf(-(((float)(~a) + 0.5f) * 0x1p-32f));
-}
-
 // CTA of DOT_THREADS: partial sums of xi^T xi, nu~^T nu~, nu~^T xi of particle
 // p over the Philox blocks of slice bx, from the Box-Muller identities: with
 // z = r (cos, sin)(pi 2u_b), r^2 = -2 log u_a, a pair adds -2 log u_a to the
@@ -957,14 +952,17 @@ __device__ __forceinline__ float log_uniform32(uint32_t a)
 //    uniforms (at most 16, each at least 2^-33, so far from underflow) and
 //    one logarithm for all of them: two FP64 operations per pair instead of a
 //    logarithm each, on the few FP64 lanes that bound this kernel.
-//  * The cross product sets only the projection coefficient a of eq.
-//    nuPerpendicular, not gamma or zeta: its terms are formed in FP32, the
-//    angle's difference in 32-bit integers, where its period is exact, and
-//    summed with their rounding errors (two-sum) until the thread's FP64 total.
-//    A term's rms error against 64 bits is 0.84e-7, 1.10e-7 when the difference
-//    was rounded to FP32 unreduced and the logarithms taken in FP64.
-// With form_r_block 4.05 ms per 1000 x 208^2 coarse points with an FP64
-// logarithm per pair and a generator per normal, 0.57 ms so.
+//  * The cross product's terms need each logarithm: as two floats
+//    (log_uniform, 2^-28), so that the product rounds to float as that of two
+//    FP64 logarithms does; square root and cosine in FP32, the angle's
+//    difference in 32-bit integers, where its period is exact; the product of
+//    the two exactly, summed as three floats (two-sums), more bits than a
+//    double.  A term's rms error against 64 bits is 0.78e-7; 1.10e-7 with FP64
+//    logarithms, the difference rounded to FP32 unreduced and an FP64 sum.
+// Bound by the FP64 lanes.  With form_r_block 4.05 ms per 1000 x 208^2 coarse
+// points with an FP64 logarithm per pair and a generator per normal, 0.57 ms
+// so; the terms added in FP64 (conversions and two operations per block) took
+// 0.1 ms more.
 __device__ __forceinline__ void rand_dots_cta(uint64_t seed, uint32_t t, uint32_t s_xi, uint32_t s_nu, int NR,
                                               double* __restrict__ partial, int nblk, int p, int bx)
 {
@@ -972,7 +970,7 @@ __device__ __forceinline__ void rand_dots_cta(uint64_t seed, uint32_t t, uint32_
     const int nq = NR / 4;                           // whole blocks
     double px = 1.0, pn = 1.0;                       // products of the u_a of xi and of nu~
     double tx = 0.0, tn = 0.0, tc = 0.0;             // terms of the last, partial block
-    float cs = 0.0f, ce = 0.0f;                      // cross product: sum and its rounding errors
+    float cs = 0.0f, ce = 0.0f, cg = 0.0f;           // cross product: its sum as three floats
     static_assert(2 * DOT_BLOCKS_PER_CTA * 33 < 1000, "the products stay normal");
     for (int b = bx * DOT_THREADS + threadIdx.x; b < nq; b += nblk * DOT_THREADS) {
         const uint4 wx = philox4x32_10(make_uint4((uint32_t)b, (uint32_t)p, t, s_xi), key);
@@ -982,12 +980,24 @@ __device__ __forceinline__ void rand_dots_cta(uint64_t seed, uint32_t t, uint32_
         const uint32_t xa[2] = {wx.x, wx.z}, xb[2] = {wx.y, wx.w}, na[2] = {wn.x, wn.z}, nb[2] = {wn.y, wn.w};
 #pragma unroll
         for (int l = 0; l < 2; ++l) {
-            const float r = sqrtf(4.0f * log_uniform32(xa[l]) * log_uniform32(na[l]));
+            float xh, xl, nh, nl;
+            log_uniform(xa[l], xh, xl);
+            log_uniform(na[l], nh, nl);
+            const float q = xh * nh;
+            const float r = sqrtf(4.0f * (q + (fmaf(xh, nh, -q) + fmaf(xh, nl, xl * nh))));
             const float c = cospif((float)(int)(nb[l] - xb[l]) * 0x1p-31f);
-            const float v = r * c, ve = fmaf(r, c, -v);
-            const float s = cs + v, bb = s - cs;
-            ce += ((cs - (s - bb)) + (v - bb)) + ve;
-            cs = s;
+            // s + e = a + b exactly
+            auto two_sum = [](float a, float b, float& s, float& e) {
+                s = a + b;
+                const float bb = s - a;
+                e = (a - (s - bb)) + (b - bb);
+            };
+            const float v = r * c;
+            float e1, e2, e3;
+            two_sum(cs, v, cs, e1);
+            two_sum(ce, e1, ce, e2);
+            two_sum(ce, fmaf(r, c, -v), ce, e3);
+            cg += e2 + e3;
         }
     }
     // a last block of 1 to 3 normals: its pairs in FP64, one per lane of one warp
@@ -1013,7 +1023,7 @@ __device__ __forceinline__ void rand_dots_cta(uint64_t seed, uint32_t t, uint32_
     __shared__ double red[3][DOT_THREADS / 32];
     const double xx = warp_sum(fma(-2.0, log(px), tx));
     const double nn = warp_sum(fma(-2.0, log(pn), tn));
-    const double nx = warp_sum(((double)cs + (double)ce) + tc);
+    const double nx = warp_sum((((double)cg + (double)ce) + (double)cs) + tc);
     __syncthreads();
     if ((threadIdx.x & 31) == 0) {
         red[0][threadIdx.x >> 5] = xx;
