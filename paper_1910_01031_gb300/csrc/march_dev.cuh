@@ -27,7 +27,11 @@
 //    difference; in x with k = f dx / (2g) and the signs of v swapped;
 //  * flux: with A = a+ / (a+ - a-) and B = -A a-, the central-upwind flux is
 //    F_R + A (F_L - F_R) + B (q_L - q_R), whose rounding errors scale with
-//    the jump over the face instead of with the flux;
+//    the jump over the face but for one at the flux's own last place (the
+//    momentum flux adds F_R last for that: added within the chain of FMAs it
+//    rounded twice there, and under a mean elevation of 30 m and more in 230 m
+//    of water a forecast's momentum was 9% further from 64 bits than with the
+//    flux as one quotient; 3 to 6% nearer so);
 //  * flux differences are scaled by dt/dy once, at the update.
 #pragma once
 #include "common.cuh"
@@ -153,7 +157,8 @@ __device__ __forceinline__ void flux(T eL, T qnL, T qtL, T eR, T qnR, T qtR, con
     // p(eta) = g eta (H + eta/2) = eta (g/2 eta + g H)
     const T mL = fma(qnL, unL, mul(eL, fma(K.g_half, eL, K.gH)));
     const T mR = fma(qnR, unR, mul(eR, fma(K.g_half, eR, K.gH)));
-    F1 = fma(B, dq, fma(A, sub(mL, mR), mR));
+    // m_R last: one rounding at its last place
+    F1 = add(mR, fma(B, dq, mul(A, sub(mL, mR))));
     F2 = mul(F0, sel(F0, mul(qtL, rL), mul(qtR, rR)));
 }
 
