@@ -408,9 +408,10 @@ cudaError_t launch_step(iewpf_ctx* ctx, int s)
 
 // Time candidate shapes of the marching kernel on the context's own problem
 // and keep the fastest: both kinds with 2 and 3 columns per lane (4 spill the
-// paired form and were never the fastest) over equal chunks of the rows (march_rows: the
-// last chunk as long as the others, down to a few rows for problems too small
-// to fill the GPU otherwise), then the warps per CTA of the best.  A probe
+// paired form and were never the fastest) over equal chunks of the rows
+// (march_rows: the last chunk as long as the others, down to a few rows for
+// problems too small to fill the GPU otherwise; no shorter ones once they take
+// half as long again as the best), then the warps per CTA of the best.  A probe
 // launch reads the current state and writes the other buffer without flipping
 // the parity, so the state is left as it was; all shapes compute identical
 // values.
@@ -425,16 +426,20 @@ int tune_stepper(iewpf_ctx* ctx)
     CK(cudaEventCreate(&b));
     float best = 1e30f;
     MarchShape best_shape = ctx->shape;
+    float ms = 0.0f;       // of the last probe
     auto probe = [&](const MarchShape& sh) -> int {
-        CK(launch_rk2_march(ctx->buf[0], ctx->buf[1], ctx->par, ctx->nsub, ctx->dtp, 0, ctx->G, sh, ctx->st));
-        CK(cudaEventRecord(a, ctx->st));
-        for (int r = 0; r < 3; ++r)
-            CK(launch_rk2_march(ctx->buf[0], ctx->buf[1], ctx->par, ctx->nsub, ctx->dtp, 0, ctx->G, sh, ctx->st));
-        CK(cudaEventRecord(b, ctx->st));
-        CK(cudaEventSynchronize(b));
-        float ms = 0.0f;
-        CK(cudaEventElapsedTime(&ms, a, b));
-        ctx->launches += 4;
+        // three launches after the first, one where that took long enough to time
+        for (int r = 0, n = 1; r < 2; ++r) {
+            CK(cudaEventRecord(a, ctx->st));
+            for (int k = 0; k < n; ++k)
+                CK(launch_rk2_march(ctx->buf[0], ctx->buf[1], ctx->par, ctx->nsub, ctx->dtp, 0, ctx->G, sh, ctx->st));
+            CK(cudaEventRecord(b, ctx->st));
+            CK(cudaEventSynchronize(b));
+            CK(cudaEventElapsedTime(&ms, a, b));
+            ctx->launches += n;
+            ms /= n;
+            n = ms > 0.3f ? 1 : 3;
+        }
         if (ms < best) {
             best = ms;
             best_shape = sh;
@@ -443,16 +448,20 @@ int tune_stepper(iewpf_ctx* ctx)
     };
     int rc = IEWPF_OK;
     for (int paired = 0; paired < 2 && !rc; ++paired)
-        for (int nc = 2; nc <= 3 && !rc; ++nc)
-            for (int th : march_rows(ctx->G.ny))
-                if ((rc = probe(MarchShape{nc, th, 4, paired}))) break;
+        for (int nc = 2; nc <= 3 && !rc; ++nc) {
+            float low = 1e30f;
+            for (int th : march_rows(ctx->G.ny)) {
+                if ((rc = probe(MarchShape{nc, th, 4, paired})) || ms > 1.5f * low) break;
+                low = std::min(low, ms);
+            }
+        }
     const MarchShape at4 = best_shape;
     for (int w : {2, 8})
         if (!rc) rc = probe(MarchShape{at4.nc, at4.TH, w, at4.paired});
     // the resident model step, 16 scheme steps a probe, against 16 of the best
     // march with the loop control of a captured forecast (5 us a scheme step)
     ctx->resident = 0;
-    float per_step = best / 3.0f + 0.005f;
+    float per_step = best + 0.005f;
     auto probe_resident = [&](int cl) -> int {
         for (int r = 0; r < 2; ++r) {
             if (r) CK(cudaEventRecord(a, ctx->st));
@@ -461,7 +470,6 @@ int tune_stepper(iewpf_ctx* ctx)
         }
         CK(cudaEventRecord(b, ctx->st));
         CK(cudaEventSynchronize(b));
-        float ms = 0.0f;
         CK(cudaEventElapsedTime(&ms, a, b));
         ctx->launches += 2;
         if (ms / 16.0f < per_step) {

@@ -786,6 +786,7 @@ cudaError_t batch_tune(BatchImpl& b, cudaStream_t st)
     cudaEventCreate(&z);
     float best = 1e30f;
     int bnc = 2, bth = 64, bw = 4, bp = 0;
+    float ms = 0.0f;       // of the last probe
     auto probe = [&](int nc, int th, int w, int paired) -> cudaError_t {
         cudaError_t r;
         if ((r = batch_set_step_shape(b, nc, th, w, paired)) != cudaSuccess) return r;
@@ -794,7 +795,6 @@ cudaError_t batch_tune(BatchImpl& b, cudaStream_t st)
         if ((r = launch_step_nc(b, st)) != cudaSuccess) return r;
         cudaEventRecord(z, st);
         cudaEventSynchronize(z);
-        float ms = 0.0f;
         cudaEventElapsedTime(&ms, a, z);
         b.launches += 2;
         if (ms < best) {
@@ -808,9 +808,14 @@ cudaError_t batch_tune(BatchImpl& b, cudaStream_t st)
     };
     // shapes as in the one-problem tuner: kinds, columns and chunks, then the warps of the best
     for (int paired = 0; paired < 2; ++paired)
-        for (int nc = 2; nc <= 3; ++nc)
-            for (int th : ths)
+        for (int nc = 2; nc <= 3; ++nc) {
+            float low = 1e30f;
+            for (int th : ths) {
                 if ((e = probe(nc, th, 4, paired)) != cudaSuccess) return e;
+                if (ms > 1.5f * low) break;
+                low = std::min(low, ms);
+            }
+        }
     {
         const int nc = bnc, th = bth, paired = bp;
         for (int w : {2, 8})

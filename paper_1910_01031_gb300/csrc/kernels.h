@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "march_rows.h"
 
 namespace iewpf {
 
@@ -79,17 +80,6 @@ struct StepArgs {
 inline bool ring(int nx, int nc) { return nx % nc == 0 && nx <= 32 * nc; }
 inline int strips(int nx, int nc) { return ring(nx, nc) ? 1 : (nx + 32 * nc - 9) / (32 * nc - 8); }
 }  // namespace march
-
-// candidate chunk lengths of ny rows: 1 to 32 equal chunks, at least 2 rows each
-inline std::vector<int> march_rows(int ny)
-{
-    std::vector<int> th;
-    for (int n : {1, 2, 3, 4, 6, 8, 16, 32}) {
-        const int t = (ny + n - 1) / n;
-        if (t >= 2 && (th.empty() || t < th.back())) th.push_back(t);
-    }
-    return th;
-}
 
 // tile shape of the register-marching scheme step: NC columns per lane, TH
 // rows per chunk, warps per CTA, and whether the two Runge-Kutta stages run
