@@ -415,19 +415,22 @@ IEWPF_API int iewpf_work(iewpf_ctx_t* ctx, int64_t* particle_substeps);
 /* Scheme-step kernel of the context (Sec. 3.1; both kinds compute the same
  * scheme, bit for bit).  kind 1: register-marching kernel with nc (2, 3 or
  * 4) columns per lane, `rows` rows per chunk and `warps` (1..8) warps per
- * CTA, using the hardware reciprocal and reciprocal square root; kind 2: the
+ * CTA, using the hardware reciprocal and square root; kind 2: the
  * same march with its two Runge-Kutta stages paired in packed f32x2
  * instructions.  Errors: EINVAL (an unknown kind or shape). */
 IEWPF_API int iewpf_set_stepper(iewpf_ctx_t* ctx, int kind, int nc, int rows, int warps);
 
-/* Autotuner: times every marching shape on the context's own problem (the
- * state is left unchanged) and keeps the fastest; shape[4] (may be NULL)
- * receives (kind, nc, rows, warps).  Runs by itself before the first
- * forecast unless iewpf_set_stepper was called.  It also times whole model
- * steps with each particle resident in the shared memory of a thread-block
- * cluster, where the grid is small enough; forecasts without drifters then
- * use them if faster (same bits; iewpf_set_stepper turns them off).
- * get_stepper reads the current shape.  Errors: EINVAL, ECUDA. */
+/* Autotuner: times marching shapes on the context's own problem (the state
+ * is left unchanged) and keeps the fastest; shape[4] (may be NULL) receives
+ * (kind, nc, rows, warps).  Tried are both kinds with 2 and 3 columns per
+ * lane and 4 warps over chunks of the grid's rows (1, 2, 3, 4, 5, 6, 8, ...
+ * equal chunks and chunks of 16, 32, ... 512 rows, until shorter ones are
+ * clearly slower), then 2 and 8 warps with the best of them.  Runs by itself
+ * before the first forecast unless iewpf_set_stepper was called.  It also
+ * times whole model steps with each particle resident in the shared memory of
+ * a thread-block cluster, where the grid is small enough; forecasts without
+ * drifters then use them if faster (same bits; iewpf_set_stepper turns them
+ * off).  get_stepper reads the current shape.  Errors: EINVAL, ECUDA. */
 IEWPF_API int iewpf_tune(iewpf_ctx_t* ctx, int* shape);
 IEWPF_API int iewpf_get_stepper(const iewpf_ctx_t* ctx, int* shape);
 
