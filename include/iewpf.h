@@ -434,6 +434,15 @@ IEWPF_API int iewpf_set_stepper(iewpf_ctx_t* ctx, int kind, int nc, int rows, in
 IEWPF_API int iewpf_tune(iewpf_ctx_t* ctx, int* shape);
 IEWPF_API int iewpf_get_stepper(const iewpf_ctx_t* ctx, int* shape);
 
+/* Resident model steps: clusters of `ctas` CTAs (2, 4 or 8) hold a particle
+ * each in forecasts without drifters; 0: all forecasts march.  set_resident
+ * keeps the march's shape and, like set_stepper, stands in for the tuner;
+ * get_resident reads what it or the tuner chose.  Same bits either way.
+ * Errors: EINVAL (NULL, another number, a grid whose slabs do not fit the
+ * clusters' shared memory or have fewer than 4 rows). */
+IEWPF_API int iewpf_set_resident(iewpf_ctx_t* ctx, int ctas);
+IEWPF_API int iewpf_get_resident(const iewpf_ctx_t* ctx, int* ctas);
+
 /* Number of kernels the context has launched so far (a service of the
  * library).  Errors: EINVAL. */
 IEWPF_API int iewpf_launch_count(const iewpf_ctx_t* ctx, int64_t* count);

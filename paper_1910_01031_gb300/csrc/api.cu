@@ -1773,6 +1773,23 @@ int iewpf_get_stepper(const iewpf_ctx_t* ctx, int* shape)
     return IEWPF_OK;
 }
 
+int iewpf_set_resident(iewpf_ctx_t* ctx, int ctas)
+{
+    if (!ctx) return IEWPF_EINVAL;
+    if (ctas != 0 && ((ctas != 2 && ctas != 4 && ctas != 8) || !resident_fits(ctx->G.nx, ctx->G.ny, ctas)))
+        return fail(ctx, IEWPF_EINVAL, "bad cluster size for resident model steps");
+    ctx->resident = ctas;
+    ctx->tuned = true;
+    return IEWPF_OK;
+}
+
+int iewpf_get_resident(const iewpf_ctx_t* ctx, int* ctas)
+{
+    if (!ctx || !ctas) return IEWPF_EINVAL;
+    *ctas = ctx->resident;
+    return IEWPF_OK;
+}
+
 int iewpf_launch_count(const iewpf_ctx_t* ctx, int64_t* count)
 {
     if (!ctx || !count) return IEWPF_EINVAL;

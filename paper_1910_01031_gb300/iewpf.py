@@ -28,7 +28,7 @@ EXPORTS = ["iewpf_create", "iewpf_destroy", "iewpf_set_state", "iewpf_get_state"
            "iewpf_batch_forecast", "iewpf_drifter_obs",
            "iewpf_pull_stencil", "iewpf_local_block", "iewpf_block_levels", "iewpf_solve_group", "iewpf_add_qhalf", "iewpf_sizes", "iewpf_stream",
            "iewpf_substeps", "iewpf_factor_info", "iewpf_launch_count", "iewpf_work", "iewpf_weights_noalloc", "iewpf_set_stepper", "iewpf_tune",
-           "iewpf_get_stepper", "drifter_forecast_errors", "iewpf_batch_create", "iewpf_batch_destroy",
+           "iewpf_get_stepper", "iewpf_set_resident", "iewpf_get_resident", "drifter_forecast_errors", "iewpf_batch_create", "iewpf_batch_destroy",
            "iewpf_batch_instance", "iewpf_batch_tune", "iewpf_batch_cycle", "iewpf_batch_stream",
            "iewpf_batch_work", "iewpf_batch_last_error", "iewpf_surrogate_create", "iewpf_surrogate_destroy",
            "iewpf_surrogate_param_count", "iewpf_surrogate_set_params", "iewpf_surrogate_get_params",
@@ -132,6 +132,8 @@ def load(build_if_needed: bool = True):
     L.iewpf_set_stepper.argtypes = [_vp, c.c_int, c.c_int, c.c_int, c.c_int]
     L.iewpf_tune.argtypes = [_vp, _ip]
     L.iewpf_get_stepper.argtypes = [_vp, _ip]
+    L.iewpf_set_resident.argtypes = [_vp, c.c_int]
+    L.iewpf_get_resident.argtypes = [_vp, _ip]
     L.iewpf_batch_create.argtypes = [c.POINTER(Params), c.POINTER(_dp), c.c_int, c.POINTER(c.c_void_p)]
     L.iewpf_batch_destroy.argtypes = [_vp]
     L.iewpf_batch_instance.argtypes = [_vp, c.c_int, c.POINTER(c.c_void_p)]
@@ -431,6 +433,15 @@ class Ensemble:
         out = np.zeros(4, np.int32)
         self._chk(self.L.iewpf_get_stepper(self.h, _ptr(out, _ip)), "get_stepper")
         return tuple(int(v) for v in out)
+
+    def set_resident(self, ctas):
+        """Model steps of forecasts without drifters resident in clusters of 2, 4 or 8 CTAs (0: marched)."""
+        self._chk(self.L.iewpf_set_resident(self.h, int(ctas)), "set_resident")
+
+    def resident(self):
+        v = ctypes.c_int()
+        self._chk(self.L.iewpf_get_resident(self.h, ctypes.byref(v)), "get_resident")
+        return v.value
 
     def work(self):
         """Particle scheme steps executed so far."""
