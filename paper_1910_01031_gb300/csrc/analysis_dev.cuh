@@ -1311,7 +1311,7 @@ struct BlockIn {
     }
     __device__ __forceinline__ void fetch(const float* rp)
     {
-        // in place: the compiler would sink the loads towards their use
+        // (volatile: issued here, ahead of the products of the block before)
         asm volatile("ld.global.f32 %0, [%1];" : "=f"(x0) : "l"(rp + i0) : "memory");
         asm volatile("ld.global.f32 %0, [%1];" : "=f"(x1) : "l"(rp + i1) : "memory");
     }

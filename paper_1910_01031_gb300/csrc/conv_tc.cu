@@ -171,12 +171,11 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmap_in, const __nv_bfloat16*
         __syncwarp();
     } else if (warp == 1) {
         // ---- MMA issuer ----
-        // the elected lane issues all products of a tile (its branch keeps the
-        // operands in uniform registers) and steps the descriptors by their
-        // lower words: with 64-bit steps in a lane == 0 branch a product took
-        // 100 cycles to issue and the tensor pipe waited (hidden layers, 256 x 256
-        // x 64 fields: 271 us, now 214 at 70% of the pipe; the last layer 225,
-        // now 146).  DRAM moves their 1.05 GB in 160 us
+        // the elected lane issues all products of a tile and steps the
+        // descriptors by their lower words: with 64-bit steps in a lane == 0
+        // branch a product took 100 cycles and the tensor pipe waited (hidden
+        // layers, 256 x 256 x 64 fields: 271 us, now 214 at 70% of the pipe; the
+        // last layer 225, now 146).  DRAM moves their 1.05 GB in 160 us
         int issued = 0;
         if (tc::elect_one()) {
             constexpr uint32_t IDESC = idesc_bf16(TC_PX, COUT);

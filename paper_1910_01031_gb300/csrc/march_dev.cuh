@@ -99,8 +99,8 @@ __device__ __forceinline__ float gmm(float x, float y, float z)
 
 __device__ __forceinline__ f2 bc(float a) { return make_float2(a, a); }
 __device__ __forceinline__ f2 add(f2 a, f2 b) { return __fadd2_rn(a, b); }
-// a - b as fma(b, -1, a), the same rounding (the compiler contracts the packed
-// subtraction instruction with a product before it)
+// a - b as fma(b, -1, a), the same rounding (with the packed subtraction
+// instruction the two kinds' results differ in some last bits)
 __device__ __forceinline__ f2 sub(f2 a, f2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
 __device__ __forceinline__ f2 mul(f2 a, f2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ f2 fma(f2 a, f2 b, f2 c) { return __ffma2_rn(a, b, c); }
@@ -389,7 +389,7 @@ __device__ __forceinline__ void march_warp(const StepArgs& a, int p, int chunk, 
     for (int it = 0; it < n_it; ++it) {
         // prefetch the next input row
         float pe[NC], pqu[NC], pqv[NC];
-        if (it + 1 < n_it) {     // (under a condition, or the compiler moves the loads down to their use)
+        if (it + 1 < n_it) {
             const float* r = S.in + (long long)yn * G.nx;
 #pragma unroll
             for (int k = 0; k < NC; ++k) {
@@ -468,7 +468,7 @@ __device__ __forceinline__ void march_warp_paired(const StepArgs& a, int p, int 
     float* o = S.out + (long long)S.y0 * G.nx;
     for (int it = 0; it < n_it; ++it) {
         float pe[NC], pqu[NC], pqv[NC];
-        if (it + 1 < n_it) {     // (under a condition, or the compiler moves the loads down to their use)
+        if (it + 1 < n_it) {
             const float* r = S.in + (long long)yn * G.nx;
 #pragma unroll
             for (int k = 0; k < NC; ++k) {
