@@ -17,6 +17,7 @@
 #include "batch.h"
 #include "kernels.h"
 #include "surrogate.h"
+#include "tc_dev.cuh"
 #include <random>
 
 namespace {
@@ -963,8 +964,9 @@ int iewpf_create(const iewpf_params_t* params, const double* mooring_xy, iewpf_c
         if ((rc = dalloc(ctx, &ctx->d_Lr, (size_t)nnz)) || (rc = dalloc(ctx, &ctx->d_Lc, (size_t)nnz))) return bail(rc);
         ctx->nnz = nnz;
         // (121 coupled moorings: 1031 us per analysis of 40 particles with a warp per
-        // particle, 1053 with the stream; 1024 of them and 100 particles: 3553 and 2768)
-        if (nobs >= kNdMinObs &&
+        // particle, 1053 with the stream; 1024 of them and 100 particles: 3553 and
+        // 2768; a layout that solves by warps needs none)
+        if (nobs >= kNdMinObs && solve_group(2 * nobs, P.n_particles, tc::sm_count()) > 1 &&
             ((rc = dalloc(ctx, &ctx->d_stream, solve_stream_bytes(2 * nobs, nnz))) ||
              launch_pack_stream(ctx->d_L, 2 * nobs, nnz, ctx->d_rowidx, ctx->d_plan, ctx->d_rdiag, ctx->d_stream,
                                 ctx->st) != cudaSuccess))
