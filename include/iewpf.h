@@ -439,7 +439,8 @@ IEWPF_API int iewpf_get_stepper(const iewpf_ctx_t* ctx, int* shape);
  * keeps the march's shape and, like set_stepper, stands in for the tuner;
  * get_resident reads what it or the tuner chose.  Same bits either way.
  * Errors: EINVAL (NULL, another number, a grid whose slabs do not fit the
- * clusters' shared memory or have fewer than 4 rows). */
+ * clusters' shared memory or have fewer than 4 rows, a device part without
+ * room for such a cluster). */
 IEWPF_API int iewpf_set_resident(iewpf_ctx_t* ctx, int ctas);
 IEWPF_API int iewpf_get_resident(const iewpf_ctx_t* ctx, int* ctas);
 

@@ -1778,6 +1778,7 @@ int iewpf_get_stepper(const iewpf_ctx_t* ctx, int* shape)
 int iewpf_set_resident(iewpf_ctx_t* ctx, int ctas)
 {
     if (!ctx) return IEWPF_EINVAL;
+    CK(cudaSetDevice(ctx->dev));
     if (ctas != 0 && ((ctas != 2 && ctas != 4 && ctas != 8) || !resident_fits(ctx->G.nx, ctx->G.ny, ctas)))
         return fail(ctx, IEWPF_EINVAL, "bad cluster size for resident model steps");
     ctx->resident = ctas;

@@ -95,7 +95,7 @@ cudaError_t launch_rk2_march(float* b0, float* b1, const int* par, const int* ns
 
 // ---- resident.cu ----------------------------------------------------------
 // one model step of every particle in one launch, a cluster of cl CTAs per
-// particle (resident_fits: whether the grid's slabs fit); n_sub from amax (or
+// particle (resident_fits: whether the grid and the device allow it); n_sub from amax (or
 // fixed) as nsub_kernel, the state rewritten in place, amax cleared, the work
 // counted.  store = 0 changes nothing (timing).
 bool resident_fits(int nx, int ny, int cl);

@@ -223,31 +223,57 @@ resident_kernel(float* __restrict__ buf0, float* __restrict__ buf1, const int* _
 
 }  // namespace
 
-// Cluster sizes that hold nx x ny: slabs of at least 4 rows whose arrays fit
-// an SM's shared memory
-bool resident_fits(int nx, int ny, int cl)
+namespace {
+
+// slabs of at least 4 rows whose arrays fit an SM's shared memory
+bool slabs_fit(int nx, int ny, int cl)
 {
     return (nx + 31) / 32 <= RS_MAX_WARPS && ny / cl >= 4 && slab_bytes(nx, ny, cl) <= kSlabBytes;
+}
+
+// the launch of clusters of cl CTAs; `at` holds its attribute
+cudaLaunchConfig_t cluster_launch(int nx, int ny, int ne, int cl, cudaStream_t st, cudaLaunchAttribute* at)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(ne * cl));
+    cfg.blockDim = dim3(32 * slab_warps(nx, slab_rows(ny, cl)));
+    cfg.dynamicSmemBytes = slab_bytes(nx, ny, cl);
+    cfg.stream = st;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = (unsigned)cl;
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+}  // namespace
+
+// Cluster sizes that hold nx x ny (slabs_fit) and find as many SMs in reach of
+// one cluster on the current device (a part of a GPU may have fewer)
+bool resident_fits(int nx, int ny, int cl)
+{
+    if (!slabs_fit(nx, ny, cl)) return false;
+    if (tc::smem_attr_once<resident_kernel>((int)kSlabBytes) != cudaSuccess) return false;
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg = cluster_launch(nx, ny, 1, cl, nullptr, &at);
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, resident_kernel, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return clusters > 0;
 }
 
 cudaError_t launch_resident(float* b0, float* b1, const int* par, float* amax, int* nsub, float* dtp, const Grid& G,
                             double courant, double dt_model, int fixed, unsigned long long* work, int* flag, int cl,
                             int store, cudaStream_t st)
 {
-    if (!resident_fits(G.nx, G.ny, cl)) return cudaErrorInvalidValue;
+    if (!slabs_fit(G.nx, G.ny, cl)) return cudaErrorInvalidValue;
     cudaError_t e = tc::smem_attr_once<resident_kernel>((int)kSlabBytes);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(G.ne * cl));
-    cfg.blockDim = dim3(32 * slab_warps(G.nx, slab_rows(G.ny, cl)));
-    cfg.dynamicSmemBytes = slab_bytes(G.nx, G.ny, cl);
-    cfg.stream = st;
     cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = (unsigned)cl;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    const cudaLaunchConfig_t cfg = cluster_launch(G.nx, G.ny, G.ne, cl, st, &at);
     return cudaLaunchKernelEx(&cfg, resident_kernel, b0, b1, par, amax, nsub, dtp, G, cl, courant, dt_model, fixed, work,
                               flag, store);
 }
