@@ -200,7 +200,7 @@ __global__ void b_soar(BatchDev B)
 }
 
 template <bool PULL, int PB, int SUB>
-__global__ void __launch_bounds__(NTHREADS, PB <= 4 ? 2 : 1) b_fine(BatchDev B)
+__global__ void __launch_bounds__(NTHREADS, 2) b_fine(BatchDev B)
 {
     constexpr int TX = qhalf::FINE_TX, TY = qhalf::FINE_TY;
     constexpr int PARTS = qhalf::fine_parts(PB, SUB);
@@ -527,7 +527,7 @@ cudaError_t batch_init(BatchImpl& b, const std::vector<BInst>& insts)
                 t += (long long)((I.G.nx + OBS_TX - 1) / OBS_TX) * ((I.G.ny + OBS_TY - 1) / OBS_TY) * ((I.G.ne + n - 1) / n);
             return t;
         },
-        tc::sm_count());
+        tc::sm_count(), 2);
     for (int i = 0; i < b.n; ++i) {
         const BInst& I = insts[i];
         const long long ne = I.G.ne;

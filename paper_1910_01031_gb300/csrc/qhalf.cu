@@ -65,8 +65,11 @@ coarse_soar_kernel(const float* __restrict__ src, const float* __restrict__ wtab
 using qhalf::FINE_TX;
 using qhalf::FINE_TY;
 
+// CTAs per SM of the form for single particles
+constexpr int FINE_PER_SM1 = 4;
+
 template <bool PULL, int PB, int SUB>
-__global__ void __launch_bounds__(NTHREADS, PB <= 4 ? 2 : 1)
+__global__ void __launch_bounds__(NTHREADS, PB == 1 ? FINE_PER_SM1 : 2)
 qhalf_fine_kernel(QhalfArgs A, Grid G, Coarse C, int cap, int k_in_smem)
 {
     extern __shared__ __align__(16) float fine_smem[];
@@ -118,7 +121,7 @@ cudaError_t launch_qhalf(const QhalfArgs& A, const Grid& G, const Coarse& C, cud
                                                                                      inner_y);
     const int tiles = ((G.nx + FINE_TX - 1) / FINE_TX) * ((G.ny + FINE_TY - 1) / FINE_TY);
     const int parts = qhalf::fine_choice(
-        [&](int n) { return (long long)tiles * ((G.ne + n - 1) / n); }, tc::sm_count());
+        [&](int n) { return (long long)tiles * ((G.ne + n - 1) / n); }, tc::sm_count(), FINE_PER_SM1);
     auto run = [&](auto pull) {
         constexpr bool P = decltype(pull)::value;
         if (parts == qhalf::fine_parts(4, 1)) return launch_fine<P, 4, 1>(A, G, C, tiles, st);

@@ -10,6 +10,7 @@
 // read-modify-write.
 #pragma once
 #include "common.cuh"
+#include "fine_choice.h"
 #include "kernels.h"
 
 namespace iewpf {
@@ -126,11 +127,13 @@ __device__ __forceinline__ void soar_rows(const float* __restrict__ src, const f
 //
 // The CTA: TY rows x two strips (the OBS_TX x OBS_TY tiles of the observation
 // lists) of fine_parts(PB, SUB) particles; four warps per strip take a group of PB
-// particles each (SUB = 1), or a quarter of the rows of one group (SUB = 4, for
-// ensembles too small to fill the GPU otherwise).
+// particles each (SUB = 1), or a quarter of the rows of one group (SUB = 4);
+// fine_choice says which.
 //
 // Bound by latency and issue with 4 particles per warp (128 registers, 16 warps
-// per SM); 8 per warp halve the stencil's loads again but also the warps.
+// per SM), by latency with one (64 registers, 32 warps: 1024^2 x 1 14.5 us, 18.5
+// with 90 registers and 16); 8 per warp halve the stencil's loads again but also
+// the warps.
 // Analysis update: the tile kernel it replaced interpolated through shared
 // memory with four barriers and then applied one observation at a time to the
 // whole tile, each particle loading the stencil anew and a barrier between
@@ -141,15 +144,7 @@ __device__ __forceinline__ void soar_rows(const float* __restrict__ src, const f
 constexpr int STRIPS = OBS_TX / 32;
 constexpr int GROUPS = NTHREADS / 32 / STRIPS;
 __host__ __device__ constexpr int fine_parts(int PB, int SUB) { return PB * (GROUPS / SUB); }
-// host: (PB, SUB) by the number of particles in a CTA, as many as leave every
-// SM a CTA: 16 (4, 1), 4 (4, 4) or 1 (1, 4); ctas(parts) counts the CTAs
-template <class F>
-inline int fine_choice(F ctas, int sms)
-{
-    for (int parts : {fine_parts(4, 1), fine_parts(4, 4)})
-        if (ctas(parts) >= sms) return parts;
-    return fine_parts(1, 4);
-}
+static_assert(fine_parts(4, 1) == 16 && fine_parts(4, 4) == 4 && fine_parts(1, 4) == 1, "the forms of fine_choice");
 
 // Dynamic shared memory of one CTA (16-byte aligned) for lists of up to cap
 // observations of `parts` particles: S d as (su, su', sv, sv') of each pair of
