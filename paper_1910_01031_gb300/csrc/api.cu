@@ -439,7 +439,7 @@ int tune_stepper(iewpf_ctx* ctx)
             CK(cudaEventElapsedTime(&ms, a, b));
             ctx->launches += n;
             ms /= n;
-            n = ms > 0.3f ? 1 : 3;
+            n = ms > 0.1f ? 1 : 3;
         }
         if (ms < best) {
             best = ms;
