@@ -47,11 +47,11 @@ UNIT = "particle*cell*step/s"
 BYTES_PER_CELL_STEP = 24          # read (eta, hu, hv) + write (eta, hu, hv), float32
 # FP32 operations of one scheme step per cell (adds, multiplies and fused
 # multiply-adds, one each; no halo), counted from the kernel's arithmetic
-SCHEME_OPS_PER_CELL_STEP = 216
+SCHEME_OPS_PER_CELL_STEP = 220
 # instructions per cell and scheme step measured by ncu at 512^2 x 100
 # (smsp__inst_executed.sum x 32 / cells), per stepper kind; of the paired
-# kind's, 125 are packed and take two dispatch slots each
-ISSUE_PER_CELL_STEP = {1: 451.0, 2: 337.0}
+# kind's, about 128 are packed and seem to take two dispatch slots each
+ISSUE_PER_CELL_STEP = {1: 455.9, 2: 336.5}
 WORKLOAD = "iewpf_cycle_1024x1024_ne1000_1521moorings"
 LEGS = ("drifters", "coupled", "batched", "batched_small", "surrogate", "one_stage", "rank_histogram")
 

@@ -172,8 +172,8 @@ rand_dots_kernel(uint64_t seed, uint32_t t, uint32_t s_xi, uint32_t s_nu, int NR
 // alpha solves are spread over many SMs and the reductions, cheap next to
 // them, repeated in each.
 // One CTA of 1024 threads, a division per series term: 144 us at 10 and 100
-// particles, 896 us at 1000; in slices, with the series by Horner, about 35 us
-// at all three (analysis of 64^2 x 10: 379 -> 272 us, of 624^2 x 1000: 26.60
+// particles, 896 us at 1000; in slices, with the series by Horner, 22 us at 10
+// and 100 and 30 us at 1000 (analysis of 64^2 x 10: 379 -> 272 us, of 624^2 x 1000: 26.60
 // -> 25.74 ms).
 __global__ void __launch_bounds__(ana::SYNC_THREADS)
 sync_alpha_kernel(const double* __restrict__ phi, const double* __restrict__ partial, int nblk, int ne, int slice,

@@ -10,17 +10,20 @@ namespace {
 // broadcast from lane 0 so that everything derived from it (particle, rows,
 // row addresses) is uniform over the warp.
 //
-// Bound by instruction issue: at 512^2 x 100 the paired form executes 337
-// warp instructions per 32 cells, of which the 125 packed ones take two
-// dispatch slots each, the scalar form 451; memory traffic is a quarter of
-// what HBM could move in that time.  Registers: 168 with 2 columns per lane (the
+// Bound by instruction issue and, with 8 to 12 warps per SM, by the latency
+// that so few hide: at 512^2 x 100 the paired form executes 336 warp
+// instructions per 32 cells of the grid (the scalar form 456), the halo's share
+// among them (3 columns per lane: 576 columns for 512, and 9 rows for every
+// chunk of 256), issues in 59% of the cycles, and about 128 of the 336 are
+// packed, which seem to take two dispatch slots each; memory traffic is a
+// quarter of what HBM could move in that time.  Registers: 168 with 2 columns per lane (the
 // bound of 384 threads), so that 12 warps share an SM; 255 with 3 columns, 8
 // warps.  Giving each stage a warp of its own (128 registers, 16 warps, rows
 // handed over in shared memory) issues in 81% of the cycles instead of 58%
 // but executes 485 instructions, and is slower (401 us).
-// One launch, start of the potential and flux forms above -> now:
-//   512^2 x 100: 394 -> 384 us; 1024^2 x 64: 1033 -> 980 us;
-//   64^2 x 640 (rows closing on a ring of 32 lanes): 75 -> 60 us
+// One launch, before the potential and flux forms of march_dev.cuh -> now:
+//   512^2 x 100: 394 -> 372 us; 1024^2 x 64: 1033 -> 992 us; 1024^2 x 1000:
+//   15.2 -> 14.1 ms; 64^2 x 640 (rows closing on a ring of 32 lanes): 75 -> 60 us
 template <int NC, bool RING, bool PAIRED>
 __global__ void __launch_bounds__(NC == 2 ? 384 : 256)
 rk2_march_kernel(march::StepArgs a, int s)
