@@ -1,12 +1,13 @@
 """Kernels that a rule or the tuner chooses between, each form made to run:
-resident model steps with every cluster size, and the grouped triangular
-sweeps with 4 and 8 particles per CTA on a factor whose widest steps exceed
-the ring of entries in shared memory."""
+resident model steps with every cluster size, the grouped triangular sweeps
+with 4 and 8 particles per CTA on a factor whose widest steps exceed the ring
+of entries in shared memory, and the solves of a layout too large for them."""
 import numpy as np
 import pytest
 
+from oracle import oracle as O
 from paper_1910_01031_gb300 import iewpf, synth
-from gpu_common import ensemble, start_state
+from gpu_common import ensemble, oracle_problem, start_state
 
 pytestmark = pytest.mark.gpu
 
@@ -79,3 +80,23 @@ def test_grouped_sweeps_over_steps_larger_than_the_ring(ne, particles_per_cta):
     d = single.assimilate(None, y)
     assert diag[0, 0] == d["w_target"] and diag[0, 1] == d["beta"] and diag[0, 2] == 0
     assert np.array_equal(batch.instances[0].get_state(), single.get_state())
+
+
+def test_layouts_larger_than_any_group():
+    """3136 moorings apart from each other (6272 unknowns: too many for a group of 4, and for a warp's vector in
+    shared memory): phi of every particle against the 2 x 2 blocks solved one by one in FP64, 1e-9."""
+    m, spacing, ne = 56, 16, 3
+    n = m * spacing + 16
+    cfg = synth.Config("edge", n, n, n_particles=ne, n_obs=m * m, obs_kind=synth.OBS_MOORING, c_omega=1)
+    assert iewpf.solve_group(2 * m * m, ne) == 1
+    cells = np.array([[8 + spacing * (k % m), 8 + spacing * (k // m)] for k in range(m * m)])
+    P = oracle_problem(cfg)
+    ens = ensemble(cfg, mooring_xy=synth.cell_positions(cfg, cells))
+    U32, U64 = start_state(cfg, ne)
+    y = synth.obs_from_state(cfg, synth.initial_particle(cfg, 77, seed=5), cells, synth.obs_noise(cfg, m * m, 0))
+    ens.set_state(U32)
+    d = ens.assimilate(None, y)
+    block = O.hqht(P, O.pull_stencil(P), [tuple(cells[0])]) + cfg.obs_sigma ** 2 * np.eye(2)
+    inn = np.asarray(O.innovations(P, U64, [tuple(c) for c in cells], y)).reshape(ne, m * m, 2)
+    ref = np.einsum("pli,ij,plj->p", inn, np.linalg.inv(block), inn)
+    np.testing.assert_allclose(d["phi"], ref, rtol=1e-9)
